@@ -14,6 +14,23 @@
 // sigma_Seg(q)^2 = sum_{i in Seg} sigma_i^2 (v_i . (q_r - c))^2 is the
 // variance of <o_seg, q_seg> over the data:
 //   lb_t = |o_r - c|^2 + |q_r - c|^2 - 2 (sum_{s<t} est_s + m sum_{s>=t} sigma_s).
+//
+// <u_s, q_s> = 2 <c_s, q_s> - (2^b - 1) sum q_s.  <c_s, q_s> of 16 vectors and
+// 4 queries at a time is a matrix product on the tensor cores (mma.sync
+// m16n8k16, FP16 operands, FP32 accumulators).  A code's bits are its A
+// operand as they stand: read as a subnormal FP16 number they are c 2^-24, so
+// decoding is the bit-plane transposition, a shift and a mask.  Each query
+// coordinate is a pair of integers, hi + lo / 4096 with |hi| <= 2048 (23 bits
+// below the query's largest coordinate), in two columns of B.  Products and
+// sums are integers (times 2^-24), which FP32 holds exactly up to 2^24: the
+// tensor core's truncating accumulation loses nothing, the subtraction of
+// the code's mean is exact too, and the inner products are as good as an FP32
+// sum of the products (errors against 64 bits measured slightly below those
+// of the per-lane FP32 sums used before).
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
 #include "saq_internal.h"
 
 namespace saq {
@@ -29,130 +46,622 @@ struct SegTable {
     SegDesc s[kMaxSeg];
 };
 
-__device__ __forceinline__ int decode(const uint64_t *planes, int words, int b, int j) {
-    int c = 0;
-    for (int p = 0; p < b; ++p) c = (c << 1) | (int)((planes[p * words + (j >> 6)] >> (j & 63)) & 1ull);
-    return c;
-}
-
-// vscale[v * nk + s] = |o_s| / (|u_s| cos_s)  (0 for an all-zero segment)
-__global__ void k_vec_scale(const uint8_t *__restrict__ codes, int64_t code_stride,
-                            const float *__restrict__ factors, int nf, int64_t n, int nk,
-                            SegTable t, int prefix_bits, float *__restrict__ vscale) {
-    const int lane = threadIdx.x & 31;
-    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (v >= n) return;
-    for (int s = 0; s < nk; ++s) {
-        const SegDesc g = t.s[s];
-        const int b = (prefix_bits > 0 && prefix_bits < g.bits) ? prefix_bits : g.bits;
-        const uint64_t *pl = reinterpret_cast<const uint64_t *>(codes + v * code_stride + g.code_off);
-        float S = 0.f;
-        for (int j = lane; j < g.len; j += 32) {
-            const float u = (float)(2 * decode(pl, g.words, b, j) - ((1 << b) - 1));
-            S = fmaf(u, u, S);
-        }
+// ------------------------------------------------------------ the queries
+// out[q * dk + j] = <M_j, q_r - c> for the rows M_j of a dk x d matrix; with
+// qn2 also |q_r - c|^2 and, into qmax (zero before), the largest |out| of each
+// query (bits of a non-negative float order as integers).  A warp computes
+// CPW columns for QB queries: its lanes split the d coordinates (the rows of
+// M are read once, coalesced, and each value meets QB centred queries in
+// shared memory), so that a single query spreads over dk warps (d = 960: 8.5
+// us; on the 128 x 128 tiles of the row projection, eight blocks, 207 us).
+constexpr int kRotK = 1024;  // coordinates of the queries staged at a time
+template <int QB, int CPW, bool V4>
+__global__ void __launch_bounds__(256)
+k_query_rot(const float *__restrict__ Q, int64_t nq, int d, const float *__restrict__ mean,
+            const float *__restrict__ M, int dk, float *__restrict__ out,
+            float *__restrict__ qn2, unsigned *__restrict__ qmax) {
+    static_assert(QB * CPW == 32 || QB * CPW == 1, "one result per lane, or one per warp");
+    __shared__ __align__(16) float qs[QB][kRotK];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t q0 = (int64_t)blockIdx.y * QB;
+    const int j0 = ((int)blockIdx.x * 8 + warp) * CPW;
+    float acc[CPW * QB];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) S += __shfl_xor_sync(0xffffffffu, S, off);
-        if (lane == 0) {
-            const float nrm = factors[v * nf + g.fidx];
-            const float cs = factors[v * nf + g.fidx + 1];
-            vscale[v * nk + s] = nrm > 0.f ? nrm / (sqrtf(S) * cs) : 0.f;
+    for (int i = 0; i < CPW * QB; ++i) acc[i] = 0.f;
+    float n2 = 0.f;
+    const bool norm = qn2 && blockIdx.x == 0 && warp < QB;
+    const float *row[CPW];
+#pragma unroll
+    for (int c = 0; c < CPW; ++c) row[c] = M + (int64_t)min(j0 + c, dk - 1) * d;
+    for (int k0 = 0; k0 < d; k0 += kRotK) {
+        const int kn = min(kRotK, d - k0);
+        if (k0) __syncthreads();
+        for (int e = threadIdx.x; e < QB * kRotK; e += 256) {
+            const int b = e / kRotK, k = e % kRotK;
+            qs[b][k] = (k < kn && q0 + b < nq) ? Q[(q0 + b) * d + k0 + k] - mean[k0 + k] : 0.f;
+        }
+        __syncthreads();
+        if (norm)
+            for (int k = lane; k < kn; k += 32) n2 = fmaf(qs[warp][k], qs[warp][k], n2);
+        if constexpr (V4) {  // d % 4 == 0: every row of M is 16-byte aligned
+            for (int k = 4 * lane; k < kn; k += 128) {
+                float4 w[CPW];
+#pragma unroll
+                for (int c = 0; c < CPW; ++c)
+                    w[c] = __ldg(reinterpret_cast<const float4 *>(row[c] + k0 + k));
+#pragma unroll
+                for (int b = 0; b < QB; ++b) {
+                    const float4 y = *reinterpret_cast<const float4 *>(&qs[b][k]);
+#pragma unroll
+                    for (int c = 0; c < CPW; ++c) {
+                        float &r = acc[c * QB + b];
+                        r = fmaf(w[c].x, y.x, r);
+                        r = fmaf(w[c].y, y.y, r);
+                        r = fmaf(w[c].z, y.z, r);
+                        r = fmaf(w[c].w, y.w, r);
+                    }
+                }
+            }
+        } else {
+            for (int k = lane; k < kn; k += 32) {
+                float w[CPW];
+#pragma unroll
+                for (int c = 0; c < CPW; ++c) w[c] = __ldg(row[c] + k0 + k);
+#pragma unroll
+                for (int b = 0; b < QB; ++b)
+#pragma unroll
+                    for (int c = 0; c < CPW; ++c) acc[c * QB + b] = fmaf(w[c], qs[b][k], acc[c * QB + b]);
+            }
+        }
+    }
+    if (norm) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, off);
+        if (lane == 0 && q0 + warp < nq) qn2[q0 + warp] = n2;
+    }
+    if constexpr (QB * CPW == 1) {
+        float s = acc[0];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0 && j0 < dk) {
+            out[q0 * dk + j0] = s;
+            if (qmax) atomicMax(qmax + q0, __float_as_uint(fabsf(s)));
+        }
+    } else {
+        // 32 sums over 32 lanes: each exchange halves the values a lane holds,
+        // and lane i ends with sum i (column i / QB, query i % QB)
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const bool up = lane & off;
+#pragma unroll
+            for (int i = 0; i < off; ++i) {
+                const float give = up ? acc[i] : acc[i + off], keep = up ? acc[i + off] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+            }
+        }
+        const int j = j0 + lane / QB;
+        const int64_t q = q0 + lane % QB;
+        const bool ok = j < dk && q < nq;
+        if (ok) out[q * dk + j] = acc[0];
+        if (qmax) {
+            unsigned mx = ok ? __float_as_uint(fabsf(acc[0])) : 0u;
+#pragma unroll
+            for (int off = QB; off < 32; off <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            if (lane < QB && q < nq) atomicMax(qmax + q, mx);
         }
     }
 }
 
-// one warp per (query, vector)
-__global__ void k_estimate(const uint8_t *__restrict__ codes, int64_t code_stride,
-                           const float *__restrict__ factors, int nf, int64_t n, int nk,
-                           SegTable t, int prefix_bits, const float *__restrict__ vscale,
-                           const float *__restrict__ qrot, int dk, const float *__restrict__ qn2,
-                           int64_t nq, float *__restrict__ dist) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= n * nq) return;
-    const int64_t q = w / n, v = w % n;
-    const float *qr = qrot + q * dk;
-    float est = 0.f;
-    for (int s = 0; s < nk; ++s) {
-        const SegDesc g = t.s[s];
-        const int b = (prefix_bits > 0 && prefix_bits < g.bits) ? prefix_bits : g.bits;
-        const uint64_t *pl = reinterpret_cast<const uint64_t *>(codes + v * code_stride + g.code_off);
-        float acc = 0.f;
-        for (int j = lane; j < g.len; j += 32) {
-            const float u = (float)(2 * decode(pl, g.words, b, j) - ((1 << b) - 1));
-            acc = fmaf(u, qr[g.off + j], acc);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        est = fmaf(acc, vscale[v * nk + s], est);
-    }
-    if (lane == 0) dist[q * n + v] = factors[v * nf] + qn2[q] - 2.f * est;
-}
-
-// sig[q * nk + s] = sigma_Seg(q) = |B_s (q_r - c)|, B_s = rows sigma_i v_i^T of
-// the segment; one warp per (query, kept segment)
-__global__ void k_query_sigma(const float *__restrict__ Q, int64_t nq, int d,
-                              const float *__restrict__ mean, const float *__restrict__ B, int nk,
-                              SegTable t, float *__restrict__ sig) {
+// sig[q * nk + s] = sigma_Seg(q) = |B_s (q_r - c)| from the rotated values
+// pc[q * dk + i] (rows sigma_i v_i^T); one warp per (query, kept segment)
+__global__ void k_query_sigma(const float *__restrict__ pc, int64_t nq, int dk, int nk,
+                              const __grid_constant__ SegTable t, float *__restrict__ sig) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= nq * nk) return;
     const int64_t q = w / nk;
     const int s = (int)(w % nk);
-    const SegDesc g = t.s[s];
-    const float *qv = Q + q * d;
+    const float *p = pc + q * dk + t.s[s].off;
     float acc = 0.f;
-    for (int i = 0; i < g.len; ++i) {
-        const float *b = B + (int64_t)(g.off + i) * d;
-        float dot = 0.f;
-        for (int k = lane; k < d; k += 32) dot = fmaf(b[k], qv[k] - mean[k], dot);
+    for (int i = lane; i < t.s[s].len; i += 32) acc = fmaf(p[i], p[i], acc);
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-        acc = fmaf(dot, dot, acc);
-    }
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) sig[q * nk + s] = sqrtf(acc);
 }
 
-// bounds[(q * n + v) * (nk + 1) + t] = lb_t; one warp per (query, vector)
-__global__ void k_estimate_staged(const uint8_t *__restrict__ codes, int64_t code_stride,
-                                  const float *__restrict__ factors, int nf, int64_t n, int nk,
-                                  SegTable t, const float *__restrict__ vscale,
-                                  const float *__restrict__ qrot, int dk,
-                                  const float *__restrict__ qn2, int64_t nq,
-                                  const float *__restrict__ qsig, float m_conf,
-                                  float *__restrict__ bounds) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= n * nq) return;
-    const int64_t q = w / n, v = w % n;
-    const float *qr = qrot + q * dk;
-    const float *sg = qsig + q * nk;
-    const float base = factors[v * nf] + qn2[q];
-    float *out = bounds + (q * n + v) * (int64_t)(nk + 1);
-    auto rest = [&](int t0) {  // m * sum_{s >= t0} sigma_s
-        float r = 0.f;
-        for (int s = t0; s < nk; ++s) r += sg[s];
-        return m_conf * r;
-    };
-    if (lane == 0) out[0] = base - 2.f * rest(0);
-    float done = 0.f;
-    for (int s = 0; s < nk; ++s) {
-        const SegDesc g = t.s[s];
-        const uint64_t *pl = reinterpret_cast<const uint64_t *>(codes + v * code_stride + g.code_off);
-        float acc = 0.f;
-        for (int j = lane; j < g.len; j += 32) {
-            const float u = (float)(2 * decode(pl, g.words, g.bits, j) - ((1 << g.bits) - 1));
-            acc = fmaf(u, qr[g.off + j], acc);
+// The exponent that brings a query's largest coordinate into [1024, 2048)
+// (0 for an all-zero query or one that is not finite, whose estimates are
+// not finite either).
+__device__ __forceinline__ int query_exponent(unsigned mx) {
+    if (mx == 0u || mx >= 0x7F800000u) return 0;
+    return min(120, 10 - ilogbf(__uint_as_float(mx)));
+}
+
+// The coordinate (of a segment of `words` 64-bit words) that element i (0..3)
+// of lane quad position t holds in K step `step` of the segment.  The lanes of
+// a quad decode 32 bits of a plane each at a time (8 steps of 16 coordinates):
+// lane t bits 32 h .. of word 4 c + t of the chunk of four words c (h = 0, 1:
+// the quad reads 32 contiguous bytes over the two), then, of two words left
+// over, bits 32 t .. of both, and of a last one 16 bits each (4 steps).
+__device__ __forceinline__ int step_coord(int words, int step, int t, int i) {
+    const int full = words >> 2, m = step & 7, c = step >> 4;
+    const int k = m >> 1, r = 2 * (m & 1) + (i >> 1), hi = i & 1;
+    if (c < full) return (4 * c + t) * 64 + ((step >> 3) & 1) * 32 + 4 * k + r + 16 * hi;
+    const int at = 256 * full;
+    if ((words & 2) && step - 16 * full < 8) return at + 32 * t + 4 * k + r + 16 * hi;
+    return at + ((words & 2) ? 128 : 0) + 16 * t + 4 * k + r + 8 * hi;
+}
+
+// B fragments of every pass: entry ((pass * steps + step) * NT + nt) * 32 +
+// lane holds the four FP16 values of column lane / 4 (query 4 (pass * NT +
+// nt) + column / 2, hi or lo part) for lane quad position lane % 4.  qsum
+// (zero before) takes the sum of each column over each segment.
+__global__ void __launch_bounds__(256)
+k_query_split(const float *__restrict__ qrot, int64_t nq, int dk, int nk,
+              const __grid_constant__ SegTable t, int steps, int NT, int64_t total,
+              const unsigned *__restrict__ qmax, uint2 *__restrict__ bfrag,
+              int *__restrict__ qsum, int64_t cols) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int lane = (int)(e & 31);
+    const int64_t f = e >> 5;
+    const int nt = (int)(f % NT);
+    const int gstep = (int)((f / NT) % steps);
+    const int64_t pass = f / NT / steps;
+    const int64_t q = 4 * (pass * NT + nt) + (lane >> 3);
+    const bool lo = (lane >> 2) & 1;
+    int s = 0, step = gstep;
+    while (s + 1 < nk && step >= 4 * t.s[s].words) step -= 4 * t.s[s++].words;
+    __half h[4];
+    int sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = step_coord(t.s[s].words, step, lane & 3, i);
+        float v = 0.f;
+        if (q < nq && c < t.s[s].len) {
+            const float y = scalbnf(qrot[q * dk + t.s[s].off + c], query_exponent(qmax[q]));
+            const float r = rintf(y);
+            v = lo ? rintf((y - r) * 4096.f) : r;
+        }
+        h[i] = __float2half_rn(v);
+        sum += (int)v;
+    }
+    uint2 o;
+    o.x = (uint32_t)__half_as_ushort(h[0]) | (uint32_t)__half_as_ushort(h[1]) << 16;
+    o.y = (uint32_t)__half_as_ushort(h[2]) | (uint32_t)__half_as_ushort(h[3]) << 16;
+    bfrag[e] = o;
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);  // total is a multiple of 32: whole warps
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    if ((lane & 3) == 0) atomicAdd(qsum + s * cols + 8 * (pass * NT + nt) + (lane >> 2), sum);
+}
+
+// ------------------------------------------------------------ the vectors
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+        "{%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ uint32_t select_bits(uint32_t m, uint32_t a, uint32_t b) {
+    return (a & m) | (b & ~m);
+}
+
+// 32 coordinates of one vector from their plane words: planes are transposed
+// by 4 x 4 bit blocks into words whose nibble j is the code (or four bits of
+// it) of bit 4 j + r, in 16 operations for 32 codes.
+__device__ __forceinline__ void transpose4(uint32_t (&w)[4]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint32_t a = w[q], b = w[q + 2];
+        w[q] = select_bits(0x33333333u, a, b << 2);
+        w[q + 2] = select_bits(0x33333333u, a >> 2, b);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+        const uint32_t a = w[q], b = w[q + 1];
+        w[q] = select_bits(0x55555555u, a, b << 1);
+        w[q + 1] = select_bits(0x55555555u, a >> 1, b);
+    }
+}
+// NP planes (4 or 8), least significant first; planes past the code's width
+// are zero.  Two widths only: eight instantiations in one switch took 190
+// registers (each alone under 80).
+template <int NP> struct Codes {
+    uint32_t even[4], odd[4];  // bytes j: the codes of bits 8 j + r and 8 j + 4 + r
+    __device__ __forceinline__ void split(const uint32_t (&p)[NP]) {
+        uint32_t l[4] = {p[0], p[1], p[2], p[3]};
+        transpose4(l);
+        if constexpr (NP == 4) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                even[r] = l[r] & 0x0F0F0F0Fu;
+                odd[r] = (l[r] >> 4) & 0x0F0F0F0Fu;
+            }
+        } else {
+            uint32_t h[4] = {p[4], p[5], p[6], p[7]};
+            transpose4(h);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                even[r] = select_bits(0x0F0F0F0Fu, l[r], h[r] << 4);
+                odd[r] = select_bits(0x0F0F0F0Fu, l[r] >> 4, h[r]);
+            }
+        }
+    }
+    // the codes of bits 4 k + r (low half) and 4 k + r + 16
+    __device__ __forceinline__ uint32_t pair(int k, int r) const {
+        return __byte_perm((k & 1) ? odd[r] : even[r], 0u, (k & 2) ? 0x4341 : 0x4240);
+    }
+    __device__ __forceinline__ uint32_t sum2(uint32_t s) const {  // s + sum c^2
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s = __dp4a(odd[r], odd[r], __dp4a(even[r], even[r], s));
+        return s;
+    }
+};
+
+struct EstArgs {
+    const uint8_t *codes;
+    int64_t code_stride;
+    const float *factors;
+    int nf;
+    int64_t n;
+    int nk, prefix_bits;
+    const uint2 *bfrag;
+    int steps;
+    const float *qn2;
+    const unsigned *qmax;
+    const int *qsum;  // per segment and B column: the sum of the column over the segment
+    int64_t cols;     // B columns of all passes
+    int64_t nq;
+    const float *qsig;  // staged: sigma of (query, segment)
+    float m_conf;
+    float *out;
+};
+
+// The K steps of one decoded 32-bit piece (NS = 8) or 16-bit one (4): A
+// fragments from the codes and NT products per step.
+template <int NP, int NT, int MT, int NS>
+__device__ __forceinline__ void run_steps(const Codes<NP> (&cd)[MT][2], const uint2 *__restrict__ b,
+                                          float (&acc)[MT][NT][4]) {
+#pragma unroll
+    for (int m = 0; m < NS; ++m) {
+        const int k = m >> 1, r = 2 * (m & 1);
+        uint32_t a[MT][4];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            a[mt][0] = cd[mt][0].pair(k, r);
+            a[mt][1] = cd[mt][1].pair(k, r);
+            a[mt][2] = cd[mt][0].pair(k, r + 1);
+            a[mt][3] = cd[mt][1].pair(k, r + 1);
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        done = fmaf(acc, vscale[v * nk + s], done);
-        if (lane == 0) out[s + 1] = base - 2.f * (done + rest(s + 1));
+        for (int nt = 0; nt < NT; ++nt) {
+            const uint2 bv = b[(m * NT + nt) * 32];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+                mma16816(acc[mt][nt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], bv.x, bv.y);
+        }
+    }
+}
+
+// Part of a plane word (or a factor) from the staged record (SM) or from
+// global memory.
+template <bool SM, class T> __device__ __forceinline__ T load_rec(const void *p) {
+    if constexpr (SM) return *static_cast<const T *>(p);
+    else return __ldg(static_cast<const T *>(p));
+}
+
+// The products of one segment of `bits` bits (its first planes; at most NP)
+// for the warp's rows (row pointers at the segment's codes).  S2 += sum c^2 and
+// S1 += sum c over the lane's coordinates.
+template <int NP, int NT, int MT, bool SM>
+__device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], int bits, int words,
+                                            int len, int t, const uint2 *__restrict__ b,
+                                            float (&acc)[MT][NT][4],
+                                            uint32_t (&S2)[MT][2], uint32_t (&S1)[MT][2]) {
+    const bool partial = (len & 63) != 0;  // bits past the end are to read as zero
+    // sum of the codes of one lane's plane words
+    auto code_sum = [](const uint32_t (&w)[NP]) {
+        uint32_t x = 0u;
+#pragma unroll
+        for (int p = NP - 1; p >= 0; --p) x = 2u * x + (uint32_t)__popc(w[p]);
+        return x;
+    };
+    const int full = words >> 2, pieces = 2 * full + ((words >> 1) & 1);
+    const uint32_t stride = (uint32_t)words * 8u;  // bytes of a plane
+    // byte offset in a plane of the lane's 32 bits of piece i
+    auto piece_at = [&](int i) -> uint32_t {
+        return i < 2 * full ? (uint32_t)((((i >> 1) * 4 + t) << 3) + ((i & 1) << 2))
+                            : (uint32_t)(32 * full + 4 * t);
+    };
+    const uint32_t last = (uint32_t)(bits - 1) * stride;  // the least significant plane
+    uint32_t nx[MT][2][NP];
+    auto fetch = [&](int i) {
+        uint32_t at = piece_at(i) + last;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            // an offset the compiler cannot split: it would keep a 64-bit
+            // pointer per row and plane in registers otherwise
+            asm volatile("" : "+r"(at));
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    nx[mt][h][p] = p < bits ? load_rec<SM, uint32_t>(rp[mt][h] + at) : 0u;
+            at -= stride;
+        }
+    };
+    if (pieces > 0) fetch(0);
+#pragma unroll 1
+    for (int i = 0; i < pieces; ++i) {
+        if (partial) {
+            const int left = len - (int)piece_at(i) * 8;
+            const uint32_t keep = left >= 32 ? ~0u : left <= 0 ? 0u : (1u << left) - 1u;
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) nx[mt][h][p] &= keep;
+        }
+        Codes<NP> cd[MT][2];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                S1[mt][h] += code_sum(nx[mt][h]);
+                cd[mt][h].split(nx[mt][h]);
+                S2[mt][h] = cd[mt][h].sum2(S2[mt][h]);
+            }
+        if (i + 1 < pieces) fetch(i + 1);
+        run_steps<NP, NT, MT, 8>(cd, b, acc);
+        b += 8 * NT * 32;
+    }
+    if (words & 1) {
+        const uint32_t at = (uint32_t)(words - 1) * 8u + 2u * (uint32_t)t;
+        const int left = len - (int)at * 8;
+        const uint32_t keep = left >= 16 ? 0xFFFFu : left <= 0 ? 0u : (1u << left) - 1u;
+        Codes<NP> cd[MT][2];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t w[NP];
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const uint32_t x =
+                        p < bits ? load_rec<SM, uint16_t>(rp[mt][h] + (at + last - p * stride)) & keep : 0u;
+                    w[p] = __byte_perm(x, 0u, 0x2120);  // byte 0 at bits 0, byte 1 at bits 16
+                }
+                S1[mt][h] += code_sum(w);
+                cd[mt][h].split(w);
+                S2[mt][h] = cd[mt][h].sum2(S2[mt][h]);
+            }
+        run_steps<NP, NT, MT, 4>(cd, b, acc);
+    }
+}
+
+// Asynchronous copies of 16, 8 or 4 bytes into shared memory.
+template <int BYTES> __device__ __forceinline__ void copy_async(void *dst, const void *src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES)
+                     : "memory");
+}
+
+// A warp's 16 code records (rows at `stride` bytes in shared memory) and
+// their factors, rows [r0, r0 + rows).
+__device__ __forceinline__ void stage_tile(const EstArgs &A, int64_t r0, int rows, uint8_t *dst,
+                                           int stride, float *fdst, int lane) {
+    const uint8_t *src = A.codes + r0 * A.code_stride;
+    const bool wide = (A.code_stride & 15) == 0;
+    const int unit = wide ? 16 : 8, per = (int)A.code_stride / unit;
+    int r = 0, c = lane;
+    for (;;) {
+        while (c >= per && r < rows) {
+            c -= per;
+            ++r;
+        }
+        if (r >= rows) break;
+        if (wide) copy_async<16>(dst + r * stride + c * 16, src + (int64_t)r * A.code_stride + c * 16);
+        else copy_async<8>(dst + r * stride + c * 8, src + (int64_t)r * A.code_stride + c * 8);
+        c += 32;
+    }
+    const float *f = A.factors + r0 * A.nf;
+    for (int e = lane; e < rows * A.nf; e += 32) copy_async<4>(fdst + e, f + e);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// A warp takes tiles of 16 MT vectors; the block's NT B columns (4 NT queries
+// of pass blockIdx.y) stay in shared memory (BS) for all of its tiles.
+// SM: the tile's code records and factors are copied to the warp's own buffer
+// in shared memory first (asynchronously, as soon as the previous tile is
+// done), so that the loads of the decode take 30 cycles instead of an L2 or
+// HBM round trip at the start of every segment; the other warps of the SM
+// cover the copy.
+// Bound by the instructions of the decode (77% of the issue slots, 68% of the
+// integer pipe; HBM 20%, tensor pipe 10% at one query): 1 query x 1M records
+// of 480 B 4,350 -> 271 us, 100 x 100K 22,600 -> 224 us (the tensor pipe 42%),
+// against a warp per (query, vector) that decoded a bit per plane and lane.
+// Measured on the way: decode to FP16 integers by two more FP16 operations
+// per pair 405 us, |u|^2 from two more products per step (their diagonals)
+// 360 us, records read from global memory by every lane 390 us.
+template <int NT, int MT, bool BS, bool STAGED, bool SM>
+__global__ void __launch_bounds__(SM ? (NT <= 4 ? 768 : 384) : 256, 1)
+k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstride) {
+    static_assert(!SM || MT == 1, "a staged tile holds 16 records");
+    extern __shared__ __align__(16) uint2 bsm[];
+    __shared__ float s_qn2[4 * NT], s_qsc[4 * NT];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const int64_t q0 = (int64_t)blockIdx.y * 4 * NT;
+    const uint2 *bg = A.bfrag + (int64_t)blockIdx.y * A.steps * NT * 32;
+    const int64_t tiles = (A.n + 16 * MT - 1) / (16 * MT), tstep = (int64_t)gridDim.x * warps;
+    int64_t tile = (int64_t)blockIdx.x * warps + warp;
+    // the warp's buffer: 16 records, then their factors
+    uint8_t *buf = reinterpret_cast<uint8_t *>(bsm + (BS ? A.steps * NT * 32 : 0)) +
+                   (SM ? warp * (16 * sstride + ((64 * A.nf + 15) & ~15)) : 0);
+    float *fbuf = reinterpret_cast<float *>(buf + 16 * sstride);
+    if (SM && tile < tiles)
+        stage_tile(A, tile * 16, (int)min((int64_t)16, A.n - tile * 16), buf, sstride, fbuf, lane);
+    if constexpr (BS)
+        for (int e = threadIdx.x; e < A.steps * NT * 16; e += blockDim.x)
+            reinterpret_cast<uint4 *>(bsm)[e] = __ldg(reinterpret_cast<const uint4 *>(bg) + e);
+    for (int e = threadIdx.x; e < 4 * NT; e += blockDim.x) {
+        const int64_t q = q0 + e;
+        s_qn2[e] = q < A.nq ? A.qn2[q] : 0.f;
+        s_qsc[e] = q < A.nq ? scalbnf(1.f, -query_exponent(A.qmax[q])) : 0.f;
+    }
+    __syncthreads();
+    const uint2 *b0 = (BS ? bsm : bg) + lane;
+    for (; tile < tiles; tile += tstep) {
+        int64_t v[MT][2];
+        const float *fac[MT][2];
+        const uint8_t *rec[MT][2];
+        if constexpr (SM) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+        }
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                v[mt][h] = tile * (16 * MT) + mt * 16 + h * 8 + g;
+                if constexpr (SM) {  // rows past n: whatever the buffer holds
+                    fac[mt][h] = fbuf + (h * 8 + g) * A.nf;
+                    rec[mt][h] = buf + (h * 8 + g) * sstride;
+                } else {
+                    const int64_t r = min(v[mt][h], A.n - 1);  // rows past n repeat the last one
+                    fac[mt][h] = A.factors + r * A.nf;
+                    rec[mt][h] = A.codes + r * A.code_stride;
+                }
+            }
+        float est[MT][NT][2];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) est[mt][nt][0] = est[mt][nt][1] = 0.f;
+        auto store = [&](int stage) {
+            // value after `stage` segments (or the distance itself)
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (v[mt][h] >= A.n) continue;
+                    const float f0 = load_rec<SM, float>(fac[mt][h]);
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        const int64_t q = q0 + 4 * nt + t;
+                        if (q >= A.nq) continue;
+                        const float base = f0 + s_qn2[4 * nt + t];
+                        const float e = est[mt][nt][h] * s_qsc[4 * nt + t];
+                        if constexpr (STAGED) {
+                            float rest = 0.f;  // m * sum_{s >= stage} sigma_s
+                            for (int s = stage; s < A.nk; ++s) rest += __ldg(A.qsig + q * A.nk + s);
+                            rest *= A.m_conf;
+                            A.out[(q * A.n + v[mt][h]) * (A.nk + 1) + stage] = base - 2.f * (e + rest);
+                        } else {
+                            A.out[q * A.n + v[mt][h]] = base - 2.f * e;
+                        }
+                    }
+                }
+        };
+        if constexpr (STAGED) store(0);
+        int step0 = 0;
+        for (int s = 0; s < A.nk; ++s) {
+            const SegDesc &sg = tab.s[s];
+            const int bits = A.prefix_bits > 0 ? min(A.prefix_bits, sg.bits) : sg.bits;
+            const uint8_t *rp[MT][2];
+            float acc[MT][NT][4];
+            uint32_t S2[MT][2], S1[MT][2];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                rp[mt][0] = rec[mt][0] + sg.code_off;
+                rp[mt][1] = rec[mt][1] + sg.code_off;
+                S2[mt][0] = S2[mt][1] = 0u;
+                S1[mt][0] = S1[mt][1] = 0u;
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
+            }
+            // the two factors of one of the lane quad's rows in each of its lanes
+            const float *fv = fac[0][0];
+#pragma unroll
+            for (int i = 1; i < 2 * MT; ++i)
+                if (t % (2 * MT) == i) fv = fac[i >> 1][i & 1];
+            const float nrm = load_rec<SM, float>(fv + sg.fidx);
+            const float cs = load_rec<SM, float>(fv + sg.fidx + 1);
+            const uint2 *b = b0 + step0 * NT * 32;
+            if (bits <= 4)  // uniform
+                run_segment<4, NT, MT, SM>(rp, bits, sg.words, sg.len, t, b, acc, S2, S1);
+            else
+                run_segment<8, NT, MT, SM>(rp, bits, sg.words, sg.len, t, b, acc, S2, S1);
+            step0 += 4 * sg.words;
+            // |u|^2 = 4 (sum c^2 - cmax sum c) + len cmax^2, the sums spread
+            // over the quad; lane t forms the scale of row t % (2 MT)
+            const int cmax = (1 << bits) - 1;
+            long long c2 = 0;
+#pragma unroll
+            for (int i = 0; i < 2 * MT; ++i) {
+                const uint32_t s2 = S2[i >> 1][i & 1], s1 = S1[i >> 1][i & 1];
+                long long x;
+                if (sg.len > 65536) {  // uniform
+                    x = (long long)s2 - (long long)cmax * s1;
+                    x += __shfl_xor_sync(0xffffffffu, x, 1);
+                    x += __shfl_xor_sync(0xffffffffu, x, 2);
+                } else {
+                    uint32_t lo = s2 - (uint32_t)cmax * s1;
+                    lo += __shfl_xor_sync(0xffffffffu, lo, 1);
+                    lo += __shfl_xor_sync(0xffffffffu, lo, 2);
+                    x = lo;
+                }
+                if (t % (2 * MT) == i) c2 = x;
+            }
+            // (modulo 2^32 |u|^2 is exact up to 66,051 coordinates of 8 bits)
+            const float S = sg.len > 65536
+                                ? (float)(4ll * c2 + (long long)sg.len * (cmax * cmax))
+                                : (float)(4u * (uint32_t)c2 + (uint32_t)sg.len * (uint32_t)(cmax * cmax));
+            const float vs = nrm > 0.f ? nrm / (sqrtf(S) * cs) : 0.f;
+            const float fc = -(float)cmax;
+            const int *qs = A.qsum + (int64_t)s * A.cols + (int64_t)blockIdx.y * 8 * NT + 2 * t;
+            float vsr[MT][2];
+#pragma unroll
+            for (int i = 0; i < 2 * MT; ++i)
+                vsr[i >> 1][i & 1] = __shfl_sync(0xffffffffu, vs, (g << 2) | i);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const int2 sum = __ldg(reinterpret_cast<const int2 *>(qs + 8 * nt));
+                const float sh = (float)sum.x, sl = (float)sum.y;
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        // <u, hi> and <u, lo>: 2 <c, .> - cmax sum
+                        const float hi = fmaf(fc, sh, acc[mt][nt][2 * h] * 0x1p25f);
+                        const float lo = fmaf(fc, sl, acc[mt][nt][2 * h + 1] * 0x1p25f);
+                        est[mt][nt][h] = fmaf(fmaf(lo, 1.f / 4096.f, hi), vsr[mt][h], est[mt][nt][h]);
+                    }
+            }
+            if constexpr (STAGED) store(s + 1);
+        }
+        if constexpr (!STAGED) store(0);
+        if constexpr (SM) {
+            __syncwarp();  // every lane is done with the buffer
+            const int64_t next = tile + tstep;
+            if (next < tiles)
+                stage_tile(A, next * 16, (int)min((int64_t)16, A.n - next * 16), buf, sstride, fbuf,
+                           lane);
+        }
     }
 }
 
 SegTable seg_table(const saq_model *m) {
-    SegTable t;
+    SegTable t{};
     for (size_t i = 0; i < m->kept.size(); ++i) {
         const KeptSeg &k = m->kept[i];
         t.s[i] = SegDesc{k.off, k.len, k.bits, k.words, k.fidx, (long long)k.code_off};
@@ -160,62 +669,247 @@ SegTable seg_table(const saq_model *m) {
     return t;
 }
 
-}  // namespace
+// K steps of 16 coordinates over all kept segments.
+int total_steps(const saq_model *m) {
+    int steps = 0;
+    for (const KeptSeg &k : m->kept) steps += 4 * k.words;
+    return steps;
+}
 
-saq_status launch_estimate_staged(const saq_model *m, const uint8_t *codes, const float *factors,
-                                  int64_t n, const float *Q, const float *Qrot, const float *qn2,
-                                  int64_t nq, float m_conf, float *vscale, float *qsig,
-                                  float *bounds, cudaStream_t s) {
-    const int nk = (int)m->kept.size();
-    if (nk > kMaxSeg) return set_error(SAQ_ERR_UNSUPPORTED, "more than %d kept segments", kMaxSeg);
-    const SegTable t = seg_table(m);
-    const int64_t cs = (int64_t)m->code_bytes;
-    {
-        LaunchTimer lt_(kKindOther, s);
-        k_vec_scale<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(codes, cs, factors, m->nf, n, nk, t, 0,
-                                                             vscale);
+constexpr size_t kEstSmemMax = 224 * 1024;  // dynamic shared memory of a block
+
+// Row stride of the staged records: 32 or 96 bytes past a multiple of 128, so
+// that the eight rows a quad column reads fall into four bank groups.
+int staged_stride(const saq_model *m) {
+    const int s = ((int)m->code_bytes + 31) / 32 * 32;
+    return s % 64 == 32 ? s : s + 32;
+}
+// Bytes of a warp's buffer (16 records and their factors).
+size_t staged_bytes(const saq_model *m) {
+    return (size_t)16 * staged_stride(m) + (((size_t)64 * m->nf + 15) & ~(size_t)15);
+}
+
+struct EstPlan {
+    int NT = 1, steps = 0;
+    int64_t passes = 1;
+    bool bs = true;  // B in shared memory (else read through the caches)
+    int warps = 0;   // staged form: warps per block (0: the form without staging)
+    int64_t cols() const { return passes * NT * 8; }
+};
+// 4 NT queries per pass: the fewest passes whose B columns fit in shared
+// memory, then the smallest form that still does them in that many.  Records
+// are staged when the buffers of at least eight warps fit beside B.
+EstPlan est_plan(const saq_model *m, int64_t nq) {
+    static const int forms[] = {1, 4, 8};
+    EstPlan p;
+    p.steps = total_steps(m);
+    const int64_t nts = (nq + 3) / 4;
+    const size_t wb = staged_bytes(m);
+    const auto choose = [&](size_t beside) {
+        int most = 0;
+        for (int f : forms)
+            if ((size_t)p.steps * f * 256 + beside <= kEstSmemMax) most = f;
+        if (!most) return false;
+        const int64_t need = (nts + (nts + most - 1) / most - 1) / ((nts + most - 1) / most);
+        for (int f : forms)
+            if (f >= need) {
+                p.NT = f;
+                break;
+            }
+        p.passes = (nts + p.NT - 1) / p.NT;
+        return true;
+    };
+    if (choose(8 * wb)) {
+        const int fit = (int)((kEstSmemMax - (size_t)p.steps * p.NT * 256) / wb);
+        p.warps = std::min(p.NT <= 4 ? 24 : 12, fit);
+    } else if (!choose(0)) {
+        p.bs = false;
+        p.NT = 1;
+        p.passes = nts;
     }
-    {
-        LaunchTimer lt_(kKindOther, s);
-        k_query_sigma<<<(unsigned)((nq * nk + 7) / 8), 256, 0, s>>>(Q, nq, m->d, m->d_mean, m->d_B,
-                                                                     nk, t, qsig);
+    return p;
+}
+
+template <int NT, int MT, bool BS, bool STAGED, bool SM>
+saq_status launch_form(const EstArgs &a, const SegTable &t, const EstPlan &p, int sstride,
+                       size_t wb, cudaStream_t s) {
+    const auto kernel = k_estimate_mma<NT, MT, BS, STAGED, SM>;
+    const int warps = SM ? p.warps : 8;
+    const size_t smem = (BS ? (size_t)a.steps * NT * 256 : 0) + (SM ? warps * wb : 0);
+    int dev = 0, sms = 0, per_sm = 0;
+    SAQ_CUDA_CHECK(cudaGetDevice(&dev));
+    SAQ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    SAQ_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kEstSmemMax));
+    SAQ_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, warps * 32, smem));
+    const int64_t tiles = (a.n + 16 * MT - 1) / (16 * MT);
+    for (int64_t p0 = 0; p0 < p.passes; p0 += 65535) {
+        const int64_t np = std::min<int64_t>(65535, p.passes - p0);
+        // the passes share the SMs; a block keeps its B columns over its tiles
+        const int64_t each = std::max<int64_t>(1, ((int64_t)sms * std::max(1, per_sm) + np - 1) / np);
+        // few tiles: as many blocks as there are SMs to take them
+        int w = warps;
+        if (SM) w = (int)std::max<int64_t>(4, std::min<int64_t>(w, (tiles + each - 1) / each));
+        w = std::min(w, warps);
+        EstArgs b = a;
+        b.bfrag += p0 * a.steps * NT * 32;
+        b.qn2 += p0 * 4 * NT;
+        b.qmax += p0 * 4 * NT;
+        b.qsum += p0 * 8 * NT;
+        if (STAGED) b.qsig += p0 * 4 * NT * a.nk;
+        b.nq -= p0 * 4 * NT;
+        b.out += p0 * 4 * NT * a.n * (STAGED ? a.nk + 1 : 1);
+        {
+            LaunchTimer lt_(kKindOther, s);
+            kernel<<<dim3((unsigned)std::min((tiles + w - 1) / w, each), (unsigned)np), w * 32, smem,
+                     s>>>(b, t, sstride);
+        }
+        note_launches();
     }
-    {
-        LaunchTimer lt_(kKindOther, s);
-        k_estimate_staged<<<(unsigned)((n * nq + 7) / 8), 256, 0, s>>>(
-            codes, cs, factors, m->nf, n, nk, t, vscale, Qrot, m->dk, qn2, nq, qsig, m_conf, bounds);
-    }
-    note_launches(3);
     SAQ_CUDA_CHECK(cudaGetLastError());
     return SAQ_OK;
 }
 
-saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float *factors,
-                           int64_t n, const float *Qrot, const float *qn2, int64_t nq,
-                           int prefix_bits, float *vscale, float *dist, cudaStream_t s) {
-    const int nk = (int)m->kept.size();
-    if (nk > kMaxSeg) return set_error(SAQ_ERR_UNSUPPORTED, "more than %d kept segments", kMaxSeg);
-    SegTable t;
-    for (int i = 0; i < nk; ++i) {
-        const KeptSeg &k = m->kept[(size_t)i];
-        t.s[i] = SegDesc{k.off, k.len, k.bits, k.words, k.fidx, (long long)k.code_off};
+template <bool STAGED>
+saq_status launch_forms(const saq_model *m, const EstArgs &a, const SegTable &t, const EstPlan &p,
+                        cudaStream_t s) {
+    const int ss = staged_stride(m);
+    const size_t wb = staged_bytes(m);
+    if (!p.bs) return launch_form<1, 1, false, STAGED, false>(a, t, p, ss, wb, s);
+    if (p.warps > 0) {
+        switch (p.NT) {
+            case 1: return launch_form<1, 1, true, STAGED, true>(a, t, p, ss, wb, s);
+            case 4: return launch_form<4, 1, true, STAGED, true>(a, t, p, ss, wb, s);
+            default: return launch_form<8, 1, true, STAGED, true>(a, t, p, ss, wb, s);
+        }
     }
-    const int64_t cs = (int64_t)m->code_bytes;
-    {
-        LaunchTimer lt_(kKindOther, s);
-        k_vec_scale<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(codes, cs, factors, m->nf, n, nk, t,
-                                                             prefix_bits, vscale);
+    switch (p.NT) {
+        case 1: return launch_form<1, 1, true, STAGED, false>(a, t, p, ss, wb, s);
+        case 4: return launch_form<4, 1, true, STAGED, false>(a, t, p, ss, wb, s);
+        default: return launch_form<8, 2, true, STAGED, false>(a, t, p, ss, wb, s);
     }
-    const int64_t warps = n * nq;
-    {
-        LaunchTimer lt_(kKindOther, s);
-        k_estimate<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(codes, cs, factors, m->nf, n, nk, t,
-                                                               prefix_bits, vscale, Qrot, m->dk, qn2,
-                                                               nq, dist);
+}
+
+// out = (Q - c) M^T (nq x dk) for a dk x d matrix, with max |out| per query.
+saq_status launch_query_rot(const saq_model *m, const float *Q, int64_t nq, const float *M,
+                            float *out, float *qn2, unsigned *qmax, cudaStream_t s) {
+    // a few queries: one column per warp, so that the rows of M spread over
+    // the chip; more: eight queries share each row read
+    const bool one = nq <= 2;
+    const int qb = one ? 1 : 8, cpw = one ? 1 : 4;
+    const unsigned gx = (unsigned)((m->dk + 8 * cpw - 1) / (8 * cpw));
+    const bool v4 = m->d % 4 == 0;
+    for (int64_t q0 = 0; q0 < nq; q0 += (int64_t)65535 * qb) {
+        const int64_t n = std::min<int64_t>(nq - q0, (int64_t)65535 * qb);
+        const dim3 grid(gx, (unsigned)((n + qb - 1) / qb));
+        const float *Qp = Q + q0 * m->d;
+        float *op = out + q0 * m->dk;
+        float *np = qn2 ? qn2 + q0 : nullptr;
+        unsigned *mp = qmax ? qmax + q0 : nullptr;
+        LaunchTimer lt_(kKindProject, s);
+        if (one && v4) k_query_rot<1, 1, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
+        else if (one) k_query_rot<1, 1, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
+        else if (v4) k_query_rot<8, 4, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
+        else k_query_rot<8, 4, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
+        note_launches();
     }
-    note_launches(2);
     SAQ_CUDA_CHECK(cudaGetLastError());
     return SAQ_OK;
+}
+
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Scratch: rotated queries, |q - c|^2, max |q_rot| and the column sums (both
+// zeroed before use), B fragments and, for the staged bounds, the basis values and sigma of (query, segment).
+struct EstScratch {
+    float *qrot, *qn2, *pc, *qsig;
+    unsigned *qmax;
+    int *qsum;
+    uint2 *bfrag;
+    size_t bytes, zero_bytes;
+};
+EstScratch est_scratch(const saq_model *m, int64_t nq, const EstPlan &p, bool staged, void *base) {
+    EstScratch r{};
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        uint8_t *q = static_cast<uint8_t *>(base) + at;
+        at += align256(bytes);
+        return q;
+    };
+    const size_t dk = (size_t)std::max(1, m->dk), q = (size_t)nq;
+    r.qrot = (float *)take(4 * q * dk);
+    r.qn2 = (float *)take(4 * q);
+    const size_t at0 = at;
+    r.qmax = (unsigned *)take(4 * q);
+    r.qsum = (int *)take(4 * (size_t)p.cols() * std::max<size_t>(1, m->kept.size()));
+    r.zero_bytes = at - at0;
+    r.bfrag = (uint2 *)take((size_t)p.passes * p.steps * p.NT * 256);
+    if (staged) {
+        r.pc = (float *)take(4 * q * dk);
+        r.qsig = (float *)take(4 * q * std::max<size_t>(1, m->kept.size()));
+    }
+    r.bytes = at;
+    return r;
+}
+
+}  // namespace
+
+size_t estimate_scratch_bytes(const saq_model *m, int64_t nq, bool staged) {
+    return est_scratch(m, nq, est_plan(m, nq), staged, nullptr).bytes;
+}
+
+saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float *factors,
+                           int64_t n, const float *Q, int64_t nq, int prefix_bits, bool staged,
+                           float m_conf, void *scratch, float *out, cudaStream_t s) {
+    const int nk = (int)m->kept.size();
+    if (nk > kMaxSeg) return set_error(SAQ_ERR_UNSUPPORTED, "more than %d kept segments", kMaxSeg);
+    const SegTable t = seg_table(m);
+    const EstPlan p = est_plan(m, nq);
+    const EstScratch w = est_scratch(m, nq, p, staged, scratch);
+    SAQ_CUDA_CHECK(cudaMemsetAsync(w.qmax, 0, w.zero_bytes, s));
+    if (nk == 0) {
+        saq_status st = launch_rownorm2(m, Q, nq, w.qn2, 1, s);
+        if (st != SAQ_OK) return st;
+    } else {
+        saq_status st = launch_query_rot(m, Q, nq, m->d_W, w.qrot, w.qn2, w.qmax, s);
+        if (st != SAQ_OK) return st;
+        const int64_t total = p.passes * p.steps * p.NT * 32;
+        {
+            LaunchTimer lt_(kKindOther, s);
+            k_query_split<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
+                w.qrot, nq, m->dk, nk, t, p.steps, p.NT, total, w.qmax, w.bfrag, w.qsum, p.cols());
+        }
+        note_launches();
+        if (staged) {
+            st = launch_query_rot(m, Q, nq, m->d_B, w.pc, nullptr, nullptr, s);
+            if (st != SAQ_OK) return st;
+            {
+                LaunchTimer lt_(kKindOther, s);
+                k_query_sigma<<<(unsigned)((nq * nk + 7) / 8), 256, 0, s>>>(w.pc, nq, m->dk, nk, t,
+                                                                             w.qsig);
+            }
+            note_launches();
+        }
+    }
+    EstArgs a;
+    a.codes = codes;
+    a.code_stride = (int64_t)m->code_bytes;
+    a.factors = factors;
+    a.nf = m->nf;
+    a.n = n;
+    a.nk = nk;
+    a.prefix_bits = prefix_bits;
+    a.bfrag = w.bfrag;
+    a.steps = p.steps;
+    a.qn2 = w.qn2;
+    a.qmax = w.qmax;
+    a.qsum = w.qsum;
+    a.cols = p.cols();
+    a.nq = nq;
+    a.qsig = w.qsig;
+    a.m_conf = m_conf;
+    a.out = out;
+    return staged ? launch_forms<true>(m, a, t, p, s) : launch_forms<false>(m, a, t, p, s);
 }
 
 }  // namespace saq

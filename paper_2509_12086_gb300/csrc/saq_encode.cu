@@ -396,26 +396,12 @@ saq_status saq_estimate_dist(const saq_model *m, const uint8_t *codes_dev,
     saq_status st = check_device(m);
     if (st != SAQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t nk = m->kept.size();
-    float *qrot = nullptr, *qn2 = nullptr, *vs = nullptr;
-    const size_t bq = sizeof(float) * (size_t)nq * std::max(1, m->dk);
-    const size_t bv = sizeof(float) * (size_t)n * std::max<size_t>(1, nk);
-    if (scratch_alloc((void **)&qrot, bq, s) != cudaSuccess ||
-        scratch_alloc((void **)&qn2, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
-        scratch_alloc((void **)&vs, bv, s) != cudaSuccess) {
-        if (qrot) cudaFreeAsync(qrot, s);
-        if (qn2) cudaFreeAsync(qn2, s);
+    void *scratch = nullptr;
+    if (scratch_alloc(&scratch, estimate_scratch_bytes(m, nq, false), s) != cudaSuccess)
         return set_error(SAQ_ERR_OOM, "scratch allocation failed");
-    }
-    // queries are rotated with the FP32 CUDA-core projection
-    st = launch_project_simt(m, Q_dev, nq, qrot, m->dk, kRowMajor, s);
-    if (st == SAQ_OK) st = launch_rownorm2(m, Q_dev, nq, qn2, 1, s);
-    if (st == SAQ_OK)
-        st = launch_estimate(m, codes_dev, factors_dev, n, qrot, qn2, nq, prefix_bits, vs,
-                             dist_dev, s);
-    cudaFreeAsync(qrot, s);
-    cudaFreeAsync(qn2, s);
-    cudaFreeAsync(vs, s);
+    st = launch_estimate(m, codes_dev, factors_dev, n, Q_dev, nq, prefix_bits, false, 0.f, scratch,
+                         dist_dev, s);
+    cudaFreeAsync(scratch, s);
     return st;
 }
 
@@ -449,27 +435,12 @@ saq_status saq_estimate_staged(const saq_model *m, const uint8_t *codes_dev,
     saq_status st = check_device(m);
     if (st != SAQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t nk = std::max<size_t>(1, m->kept.size());
-    float *qrot = nullptr, *qn2 = nullptr, *vs = nullptr, *qsig = nullptr;
-    const size_t bq = sizeof(float) * (size_t)nq * std::max(1, m->dk);
-    if (scratch_alloc((void **)&qrot, bq, s) != cudaSuccess ||
-        scratch_alloc((void **)&qn2, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
-        scratch_alloc((void **)&vs, sizeof(float) * (size_t)n * nk, s) != cudaSuccess ||
-        scratch_alloc((void **)&qsig, sizeof(float) * (size_t)nq * nk, s) != cudaSuccess) {
-        if (qrot) cudaFreeAsync(qrot, s);
-        if (qn2) cudaFreeAsync(qn2, s);
-        if (vs) cudaFreeAsync(vs, s);
+    void *scratch = nullptr;
+    if (scratch_alloc(&scratch, estimate_scratch_bytes(m, nq, true), s) != cudaSuccess)
         return set_error(SAQ_ERR_OOM, "scratch allocation failed");
-    }
-    st = launch_project_simt(m, Q_dev, nq, qrot, m->dk, kRowMajor, s);
-    if (st == SAQ_OK) st = launch_rownorm2(m, Q_dev, nq, qn2, 1, s);
-    if (st == SAQ_OK)
-        st = launch_estimate_staged(m, codes_dev, factors_dev, n, Q_dev, qrot, qn2, nq, m_conf, vs,
-                                    qsig, bounds_dev, s);
-    cudaFreeAsync(qrot, s);
-    cudaFreeAsync(qn2, s);
-    cudaFreeAsync(vs, s);
-    cudaFreeAsync(qsig, s);
+    st = launch_estimate(m, codes_dev, factors_dev, n, Q_dev, nq, 0, true, m_conf, scratch,
+                         bounds_dev, s);
+    cudaFreeAsync(scratch, s);
     return st;
 }
 

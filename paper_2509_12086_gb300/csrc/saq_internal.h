@@ -229,15 +229,13 @@ struct EncodeJob {
 // as for launch_project_tc; queue: two device ints, the launches' work
 // counters (zeroed here on s before the launches).
 saq_status encode_grouped(const EncodeJob *jobs, int njobs, cudaStream_t s, int *err, int *queue);
-// Estimator.
-saq_status launch_estimate_staged(const saq_model *m, const uint8_t *codes, const float *factors,
-                                  int64_t n, const float *Q, const float *Qrot, const float *qn2,
-                                  int64_t nq, float m_conf, float *vscale, float *qsig,
-                                  float *bounds, cudaStream_t s);
-saq_status launch_estimate(const saq_model *m, const uint8_t *codes,
-                           const float *factors, int64_t n, const float *Qrot,
-                           const float *qn2, int64_t nq, int prefix_bits,
-                           float *vscale, float *dist, cudaStream_t s);
+// Estimator (k_estimate.cu): distances (staged = false, out nq x n) or the
+// multi-stage bounds (out nq x n x (kept segments + 1)) of queries Q, with a
+// scratch of estimate_scratch_bytes.
+size_t estimate_scratch_bytes(const saq_model *m, int64_t nq, bool staged);
+saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float *factors,
+                           int64_t n, const float *Q, int64_t nq, int prefix_bits, bool staged,
+                           float m_conf, void *scratch, float *out, cudaStream_t s);
 // Fit kernels (FP64).
 saq_status launch_mean_f64(const float *X, int64_t n, int d, double *mean,
                            double *partial, int nsplit, cudaStream_t s);
