@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libsaq.so")
 BUILD = os.path.join(ROOT, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["saq_host.cpp", "saq_encode.cu", "k_simt.cu", "k_caq1.cu", "k_estimate.cu",
+SOURCES = ["saq_host.cpp", "saq_encode.cu", "k_simt.cu", "k_caq1.cu", "k_caq_scan.cu", "k_estimate.cu",
            "k_fit.cu", "k_tc.cu", "saq_noalloc.cu", "saq_ingest.cu"]
 
 
@@ -35,7 +35,8 @@ def _flags():
 def _compile(src):
     obj = os.path.join(BUILD, os.path.basename(src) + ".o")
     srcp = os.path.join(CSRC, src)
-    deps = [srcp, os.path.join(CSRC, "saq_internal.h"), os.path.join(ROOT, "include", "saq.h")]
+    deps = [srcp, os.path.join(CSRC, "saq_internal.h"),
+            os.path.join(CSRC, "caq_launch.h"), os.path.join(ROOT, "include", "saq.h")]
     if os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
         return obj, ""
     cmd = [_nvcc()] + _flags() + ["-x", "cu", "-c", srcp, "-o", obj]

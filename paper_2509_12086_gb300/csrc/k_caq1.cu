@@ -30,7 +30,7 @@
 #include <algorithm>
 #include <atomic>
 
-#include "saq_internal.h"
+#include "caq_launch.h"
 
 namespace saq {
 
@@ -40,37 +40,6 @@ constexpr int kU = 8;  // loads in flight per lane in every pass
 // the most dynamic shared memory a quantize block takes for its codes (at
 // least three blocks of 256 threads per SM)
 constexpr size_t kCaqSmemMax = 72 * 1024;
-constexpr int kMaxSeg = 64;
-
-struct Seg {
-    int off, len, bits, words, fidx;
-    long long code_off;
-};
-struct SegTable {
-    Seg s[kMaxSeg];
-    int order[kMaxSeg];  // segments by decreasing length: long work starts first
-};
-// One model's rows of a launch: its interleaved projected rows, byte-code
-// scratch, v_max and outputs.
-struct CaqGroup {
-    const float *Oi;
-    int64_t n;
-    int dk, nseg, rounds, nf;
-    uint8_t *cs;
-    const float *vmax;
-    uint8_t *codes;
-    int64_t code_stride;
-    float *factors;
-    SegTable t;
-};
-// A launch over G models: global warp w belongs to the group g with
-// warp_start[g] <= w < warp_start[g + 1] (ngroups <= G).
-template <int G> struct CaqBatch {
-    int ngroups;
-    int64_t warp_start[G + 1];
-    CaqGroup g[G];
-};
-
 // Where a lane keeps its vector-segment's codes during the adjustment.  Every
 // access is by batches of kU = 8 coordinates starting at a multiple of 8,
 // through a batch state held in registers:
@@ -635,8 +604,6 @@ __global__ void k_interleave(const float *__restrict__ O, int64_t ldo, int64_t n
 
 }  // namespace
 
-namespace {
-
 saq_status make_group(const CaqJob &j, CaqGroup *g) {
     const saq_model *m = j.m;
     const int nk = (int)m->kept.size();
@@ -663,6 +630,8 @@ saq_status make_group(const CaqJob &j, CaqGroup *g) {
     g->factors = j.factors;
     return SAQ_OK;
 }
+
+namespace {
 
 // 32-bit words per lane of the shared-memory code store for model m: its
 // largest segment's, at 1, 2, 4 or 8 bits per code (B = 1, 2, 3-4, 5-8),
@@ -704,8 +673,12 @@ std::atomic<uint64_t> g_caq1_sm_ready{0}, g_caq1_grouped_sm_ready{0};
 saq_status launch_caq1(const saq_model *m, const float *Oi, int64_t n, uint8_t *cs,
                        const float *vmax, uint8_t *codes, float *factors, cudaStream_t s) {
     if (n <= 0 || m->kept.empty()) return SAQ_OK;
+    const CaqJob job{m, Oi, n, cs, vmax, codes, factors};
+    bool ran = false;
+    saq_status scan = launch_caq_scan(&job, 1, s, &ran);
+    if (scan != SAQ_OK || ran) return scan;
     CaqGroup g;
-    saq_status st = make_group(CaqJob{m, Oi, n, cs, vmax, codes, factors}, &g);
+    saq_status st = make_group(job, &g);
     if (st != SAQ_OK) return st;
     const int64_t warps = (n + 31) / 32 * g.nseg;
     const int64_t blocks = (warps + 7) / 8;
@@ -734,6 +707,9 @@ saq_status launch_caq1(const saq_model *m, const float *Oi, int64_t n, uint8_t *
 saq_status launch_caq1_grouped(const CaqJob *jobs, int njobs, int *queue, cudaStream_t s) {
     if (njobs < 1 || njobs > kMaxGroups)
         return set_error(SAQ_ERR_INVALID, "1..%d models per grouped launch", kMaxGroups);
+    bool ran = false;
+    saq_status scan = launch_caq_scan(jobs, njobs, s, &ran);
+    if (scan != SAQ_OK || ran) return scan;
     CaqBatch<kMaxGroups> b;
     b.ngroups = 0;
     b.warp_start[0] = 0;
