@@ -56,19 +56,14 @@ k_caq_scan(const __grid_constant__ CaqBatch<G> batch) {
 
     const int64_t g32 = r0 >> 5;
     const int sub = (int)(r0 & 31);
-    if (tid < R)
-        st[3 * R + tid] = tid < nv ? __ldg(P.vmax + ((g32 * P.nseg + si) << 5) + sub + tid) : 0.f;
-    __syncthreads();
     // rows into shared memory and the initial codes (Eq. find_nearest_code)
     {
         const int rr = tid % R;
-        const float vmax = st[3 * R + rr];
-        const bool live = vmax > 0.f;
-        const float inv_delta = live ? (float)(1 << (B - 1)) / vmax : 0.f;
-        const float off_c = vmax * inv_delta;
-        const float *src = P.Oi + ((g32 * P.dk + sg.off) << 5) + sub + rr;
         if (rr < nv) {
-            constexpr int kB = 8;  // loads in flight per thread
+            constexpr int kB = 8;
+            const float *src = P.Oi + ((g32 * P.dk + sg.off) << 5) + sub + rr;
+            const float vmax = __ldg(P.vmax + ((g32 * P.nseg + si) << 5) + sub + rr);
+            float inv_delta = 0.f, off_c = 0.f;
             for (int i0 = tid / R; i0 < len; i0 += 32 * kB) {
                 float x[kB];
 #pragma unroll
@@ -76,11 +71,16 @@ k_caq_scan(const __grid_constant__ CaqBatch<G> batch) {
                     const int i = i0 + 32 * k;
                     x[k] = i < len ? __ldg(src + ((int64_t)i << 5)) : 0.f;
                 }
+                if (i0 == tid / R) {  // v_max has come with the first rows
+                    inv_delta = vmax > 0.f ? (float)(1 << (B - 1)) / vmax : 0.f;
+                    off_c = vmax * inv_delta;
+                    if (tid < R) st[3 * R + tid] = vmax;
+                }
 #pragma unroll
                 for (int k = 0; k < kB; ++k) {
                     const int i = i0 + 32 * k;
                     if (i >= len) break;
-                    const float v = live ? x[k] : 0.f;
+                    const float v = vmax > 0.f ? x[k] : 0.f;
                     const float cf = fminf(fmaxf(floorf(fmaf(v, inv_delta, off_c)), 0.f), cmaxf);
                     xs[i * RS + rr] = v;
                     us[i * RS + rr] = fmaf(2.f, cf, -cmaxf);

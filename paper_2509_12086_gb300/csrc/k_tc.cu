@@ -728,7 +728,7 @@ struct ProjGroup {
     float *O, *norms, *vmax;
     int *err;
     int64_t n, nstride, ldo;
-    int dk, npass, np, nkb, il;
+    int dk, npass, np, sub, nkb, il;  // npass passes of np columns, `sub` to a stored W pass
     float x_scale, norm_limit;
     SegCols segc;
 };
@@ -875,7 +875,8 @@ __device__ __forceinline__ void proj_persistent(const ProjBatch &batch, int *que
                 // reference would be repeated after every asm with a memory
                 // clobber in the loop
                 const uint8_t *wt0 = P.wt0, *wt1 = P.wt1;
-                const int np = P.np;
+                const int np = P.np, sub = P.sub;
+                const int wp = tr.pass / sub, ws = tr.pass % sub;
                 asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)tmxp) : "memory");
                 const uint32_t tx =
                     (uint32_t)C::XBOX * kXBox + (uint32_t)C::NB * (uint32_t)np * 64u;
@@ -901,7 +902,7 @@ __device__ __forceinline__ void proj_persistent(const ProjBatch &batch, int *que
                     for (int bx = 0; bx < C::XBOX; ++bx)
                         tma_load_2d(st + bx * kXBox, tmxp, kb * C::BK + bx * 32, row0, &full[s]);
                     uint8_t *bs = st + b_offset<MODE>();
-                    const int64_t wo = ((int64_t)tr.pass * nkb + kb) * np * 64;
+                    const int64_t wo = (((int64_t)wp * nkb + kb) * sub + ws) * np * 64;
                     bulk_load(bs, wt0 + wo, (uint32_t)np * 64u, &full[s]);
                     if (C::NB == 2) bulk_load(bs + kBTile, wt1 + wo, (uint32_t)np * 64u, &full[s]);
                     if (kb + kPrefetch < nkb)
@@ -1252,6 +1253,30 @@ std::vector<T> tile_operand(const std::vector<T> &w, int dkpad, int dpad, int np
 // Role-wait bound of the next launches (saq_set_wait_limit).
 std::atomic<uint64_t> g_wait_ns{kWaitNs};
 
+// SMs of the current device (one projection CTA each).
+int sm_count() {
+    static std::atomic<int> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev < 64 && cached[dev].load() > 0) return cached[dev].load();
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 1;
+    if (dev < 64) cached[dev].store(sms);
+    return sms;
+}
+
+// Parts that a launch of `tiles` tiles splits every column pass into, so that
+// a few row tiles spread over more SMs: at most four (48 columns of 192; the
+// K loop of one tile is then bound by the copy and conversion of X, 24 ->
+// 21 us at d = 960, 52 -> 47 us at d = 3072; 16-column parts ran slower, 30 us).
+int split_passes(int64_t tiles, int np) {
+    int sub = 1;
+    for (int k = 2; k <= 4; ++k)
+        if (np % (16 * k) == 0 && np / k >= 32 && tiles * k <= sm_count()) sub = k;
+    return sub;
+}
+
 template <int MODE> saq_status launch_mode(const saq_model *m, const float *X, int64_t n,
                                            float *O, int64_t ldo, int layout, float *norms,
                                            int64_t ns, float *vmax, int *err, cudaStream_t s) {
@@ -1417,12 +1442,12 @@ namespace {
 template <int MODE>
 saq_status launch_persistent_single(const saq_model *m, const float *X, int64_t n, float *O,
                                     int64_t ldo, int il, float *norms, int64_t ns, float *vmax,
-                                    int *err, bool db, cudaStream_t s);
+                                    int *err, bool db, int *queue, cudaStream_t s);
 }  // namespace
 
 saq_status launch_project_tc(const saq_model *m, const float *X, int64_t n, float *O,
                              int64_t ldo, int layout, float *norms2, int64_t norms_stride,
-                             float *vmax, int *err, cudaStream_t s) {
+                             float *vmax, int *err, int *queue, cudaStream_t s) {
     if (n <= 0) return SAQ_OK;
     if (((uintptr_t)X & 15u) != 0) return set_error(SAQ_ERR_INVALID, "X not 16-byte aligned");
     if (m->kept.size() > 64) return set_error(SAQ_ERR_UNSUPPORTED, "more than 64 kept segments");
@@ -1431,7 +1456,7 @@ saq_status launch_project_tc(const saq_model *m, const float *X, int64_t n, floa
             // the persistent kernel (start-up and CTA changes hidden: 1.8%
             // faster than a CTA per tile at d = 960)
             return launch_persistent_single<kSplit>(m, X, n, O, ldo, layout == kInterleaved ? 1 : 0,
-                                                    norms2, norms_stride, vmax, err, false, s);
+                                                    norms2, norms_stride, vmax, err, false, queue, s);
         case SAQ_PREC_BF16:
             // the double-buffered persistent kernel where the model's passes
             // allow it, else a CTA per tile (the persistent form without the
@@ -1439,13 +1464,13 @@ saq_status launch_project_tc(const saq_model *m, const float *X, int64_t n, floa
             if (static_cast<const TcExtra *>(m->tc.extra)->db)
                 return launch_persistent_single<kBF16>(m, X, n, O, ldo,
                                                        layout == kInterleaved ? 1 : 0, norms2,
-                                                       norms_stride, vmax, err, true, s);
+                                                       norms_stride, vmax, err, true, queue, s);
             return launch_mode<kBF16>(m, X, n, O, ldo, layout, norms2, norms_stride, vmax, err, s);
         case SAQ_PREC_FP8:
             if (static_cast<const TcExtra *>(m->tc.extra)->db)
                 return launch_persistent_single<kFP8>(m, X, n, O, ldo,
                                                       layout == kInterleaved ? 1 : 0, norms2,
-                                                      norms_stride, vmax, err, true, s);
+                                                      norms_stride, vmax, err, true, queue, s);
             return launch_mode<kFP8>(m, X, n, O, ldo, layout, norms2, norms_stride, vmax, err, s);
     }
     return set_error(SAQ_ERR_INVALID, "tensor-core operands not built");
@@ -1455,7 +1480,7 @@ namespace {
 // Operands and outputs of model m's rows X (n) as one group of a persistent
 // launch (interleaved output with v_max, |x - c|^2 into norms).
 template <int MODE>
-saq_status fill_group(ProjGroup *g, const ProjJob &j, int64_t ldo, int il) {
+saq_status fill_group(ProjGroup *g, const ProjJob &j, int64_t ldo, int il, int sub) {
     const saq_model *m = j.m;
     const TcExtra *ex = static_cast<const TcExtra *>(m->tc.extra);
     saq_status st = make_map(&g->tmx, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, j.X, (uint64_t)m->d,
@@ -1474,26 +1499,14 @@ saq_status fill_group(ProjGroup *g, const ProjJob &j, int64_t ldo, int il) {
     g->ldo = ldo;
     g->il = il;
     g->dk = m->dk;
-    g->npass = ex->npass;
-    g->np = ex->np;
+    g->sub = sub;
+    g->npass = ex->npass * sub;
+    g->np = ex->np / sub;
     g->nkb = m->tc.d_pad / Cfg<MODE>::BK;
     g->x_scale = ex->x_scale;
     g->norm_limit = MODE == kSplit ? 65504.f * 65504.f : INFINITY;
     g->segc = seg_cols(m);
     return SAQ_OK;
-}
-
-// SMs of the current device (one persistent CTA each).
-int sm_count() {
-    static std::atomic<int> cached[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (dev < 64 && cached[dev].load() > 0) return cached[dev].load();
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 1;
-    if (dev < 64) cached[dev].store(sms);
-    return sms;
 }
 
 // The batch's tiles on one persistent CTA per SM (at most one per tile), taken
@@ -1541,42 +1554,50 @@ saq_status launch_grouped_mode(const ProjJob *jobs, int njobs, int *queue, cudaS
     b.tile_start[0] = 0;
     int dpad_max = 0;
     bool db = true;
+    int64_t all = 0;  // whole column passes of the batch
+    for (int i = 0; i < njobs; ++i)
+        if (jobs[i].n > 0 && jobs[i].m->dk > 0)
+            all += (jobs[i].n + kBM - 1) / kBM * static_cast<const TcExtra *>(jobs[i].m->tc.extra)->npass;
     for (int i = 0; i < njobs; ++i) {
         const ProjJob &j = jobs[i];
         const saq_model *m = j.m;
         if (j.n <= 0 || m->dk == 0) continue;
         const TcExtra *ex = static_cast<const TcExtra *>(m->tc.extra);
         db = db && ex->np <= (int)kAccDb;
-        saq_status st = fill_group<MODE>(&b.g[b.ngroups], j, m->dk, 1);
+        saq_status st = fill_group<MODE>(&b.g[b.ngroups], j, m->dk, 1, split_passes(all, ex->np));
         if (st != SAQ_OK) return st;
         dpad_max = std::max(dpad_max, m->tc.d_pad);
-        b.tile_start[b.ngroups + 1] = b.tile_start[b.ngroups] + (j.n + kBM - 1) / kBM * ex->npass;
+        b.tile_start[b.ngroups + 1] =
+            b.tile_start[b.ngroups] + (j.n + kBM - 1) / kBM * b.g[b.ngroups].npass;
         ++b.ngroups;
     }
     if (b.ngroups == 0) return SAQ_OK;
-    const int64_t tiles = b.tile_start[b.ngroups];
-    if (tiles > 0x7FFFFFFF) return set_error(SAQ_ERR_UNSUPPORTED, "too many rows in one call");
+    if (b.tile_start[b.ngroups] > 0x7FFFFFFF)
+        return set_error(SAQ_ERR_UNSUPPORTED, "too many rows in one call");
     return launch_persistent<MODE>(b, dpad_max, queue, db, s);
 }
 
-// One model's rows on the persistent kernel (db: the double-buffered one),
-// with a work counter of its own from the stream-ordered pool (freed after
-// the launch on s).
+// One model's rows on the persistent kernel (db: the double-buffered one).
+// The work counter: none for at most a tile per SM, else `queue` (zero at
+// launch), or one of its own from the stream-ordered pool.
 template <int MODE>
 saq_status launch_persistent_single(const saq_model *m, const float *X, int64_t n, float *O,
                                     int64_t ldo, int il, float *norms, int64_t ns, float *vmax,
-                                    int *err, bool db, cudaStream_t s) {
+                                    int *err, bool db, int *queue, cudaStream_t s) {
     const TcExtra *ex = static_cast<const TcExtra *>(m->tc.extra);
     ProjBatch b;
     memset(&b, 0, sizeof(b));
     b.ngroups = 1;
     b.wait_ns = g_wait_ns.load();
-    saq_status st =
-        fill_group<MODE>(&b.g[0], ProjJob{m, X, n, O, norms, ns, vmax, err}, ldo, il);
+    const int64_t rt = (n + kBM - 1) / kBM;
+    saq_status st = fill_group<MODE>(&b.g[0], ProjJob{m, X, n, O, norms, ns, vmax, err}, ldo, il,
+                                     split_passes(rt * ex->npass, ex->np));
     if (st != SAQ_OK) return st;
     b.tile_start[0] = 0;
-    b.tile_start[1] = (n + kBM - 1) / kBM * ex->npass;
-    int *queue = nullptr;
+    b.tile_start[1] = rt * b.g[0].npass;
+    if (b.tile_start[1] <= sm_count())
+        return launch_persistent<MODE>(b, m->tc.d_pad, nullptr, db, s);
+    if (queue) return launch_persistent<MODE>(b, m->tc.d_pad, queue, db, s);
     if (scratch_alloc((void **)&queue, 256, s) != cudaSuccess)
         return set_error(SAQ_ERR_OOM, "work counter allocation failed");
     st = SAQ_OK;

@@ -72,10 +72,15 @@ saq_status project_rows(const saq_model *m, const float *X, int64_t n, float *O,
                         int layout, float *norms, int64_t nstride, float *vmax, cudaStream_t s,
                         int *err) {
     if (use_tc(m)) {
-        if (vmax && layout == kInterleaved)
-            SAQ_CUDA_CHECK(cudaMemsetAsync(vmax, 0, sizeof(float) * (size_t)((n + 31) / 32 * 32) *
-                                                       m->kept.size(), s));
-        return launch_project_tc(m, X, n, O, ldo, layout, norms, nstride, vmax, err, s);
+        // one reset for v_max and the work counter ahead of it (the end of the
+        // byte scratch, which the quantizer writes only after the projection)
+        int *queue = nullptr;
+        if (vmax && layout == kInterleaved) {
+            queue = reinterpret_cast<int *>(vmax) - 4;
+            SAQ_CUDA_CHECK(cudaMemsetAsync(queue, 0, 16 + sizeof(float) * (size_t)((n + 31) / 32 * 32) *
+                                                              m->kept.size(), s));
+        }
+        return launch_project_tc(m, X, n, O, ldo, layout, norms, nstride, vmax, err, queue, s);
     }
     saq_status st = launch_project_simt(m, X, n, O, ldo, layout, s);
     if (st != SAQ_OK) return st;

@@ -130,10 +130,13 @@ saq_status launch_project_simt(const saq_model *m, const float *X, int64_t n,
 // segment, max |o| into vmax (interleaved like O: [(row/32) * nk + s] * 32 +
 // row % 32; the caller zeroes it first).
 // err: the device error word the launch raises (bounded waits that gave up,
-// input rows out of range); NULL selects the model's own word.
+// input rows out of range); NULL selects the model's own word.  queue: a device
+// work counter that is zero at launch, or NULL (the launch allocates one if
+// it needs it).
 saq_status launch_project_tc(const saq_model *m, const float *X, int64_t n,
                              float *O, int64_t ldo, int layout, float *norms2,
-                             int64_t norms_stride, float *vmax, int *err, cudaStream_t s);
+                             int64_t norms_stride, float *vmax, int *err, int *queue,
+                             cudaStream_t s);
 SegCols seg_cols(const saq_model *m);
 // One model's rows of a grouped projection launch (interleaved output, v_max
 // zeroed by the caller, |x - c|^2 into norms[i * nstride]).
@@ -199,7 +202,8 @@ saq_status launch_interleave(const float *O, int64_t ldo, int64_t n, int dk, flo
 // (FP32) followed by the byte code scratch (saq_encode.cu).
 size_t encode_scratch_bytes(const saq_model *m, int64_t rows);
 // Projection of rows [0, n) (saq_encode.cu); vmax as for launch_project_tc
-// (may be NULL).
+// (may be NULL; zeroed here).  With a vmax the 16 bytes before it belong to
+// the caller's scratch and hold the projection's work counter.
 saq_status project_rows(const saq_model *m, const float *X, int64_t n, float *O, int64_t ldo,
                         int layout, float *norms, int64_t nstride, float *vmax, cudaStream_t s,
                         int *err = nullptr);
