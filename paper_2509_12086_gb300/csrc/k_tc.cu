@@ -44,6 +44,8 @@
 //           a third of the MMAs, and the epilogue adds the two in FP32;
 //   kBF16   one BF16 product;
 //   kFP8    one E4M3 product (kind::f8f6f4), per-segment scales on W.
+// Large FP32 batches run on pairs of SMs, two CTAs to a tile of 256 rows (see
+// proj_pair); the rest is as above.
 // All waits are bounded (about 2 s); a timed-out wait raises an error flag,
 // every role leaves its loop, in-flight copies and MMAs are drained, TMEM is
 // freed and the kernel returns.
@@ -355,8 +357,9 @@ __device__ __forceinline__ uint32_t swz128(int r, int c) {
 
 // One K block of one tile row: the row's staged X values (stage st, row r)
 // centred and scaled with one FMA against -c * s (mk), converted into the A
-// operand words (split: hi in wa, lo in wl), and their squares added to nrm.
-template <int MODE>
+// operand words (split: hi in wa, lo in wl), and with NORM their squares added
+// to nrm.
+template <int MODE, bool NORM>
 __device__ __forceinline__ void convert_block(const uint8_t *st, const float *mk, int r,
                                               float x_scale, float &nrm, uint32_t (&wa)[16],
                                               uint32_t (&wl)[16]) {
@@ -374,8 +377,10 @@ __device__ __forceinline__ void convert_block(const uint8_t *st, const float *mk
                 const float4 m = *reinterpret_cast<const float4 *>(mk + ac * 16 + e * 4);
                 const float y0 = fmaf(x.x, x_scale, m.x), y1 = fmaf(x.y, x_scale, m.y);
                 const float y2 = fmaf(x.z, x_scale, m.z), y3 = fmaf(x.w, x_scale, m.w);
-                nrm = fmaf(y0, y0, nrm); nrm = fmaf(y1, y1, nrm);
-                nrm = fmaf(y2, y2, nrm); nrm = fmaf(y3, y3, nrm);
+                if (NORM) {
+                    nrm = fmaf(y0, y0, nrm); nrm = fmaf(y1, y1, nrm);
+                    nrm = fmaf(y2, y2, nrm); nrm = fmaf(y3, y3, nrm);
+                }
                 const __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(
                     make_float2(y0, y1), __NV_SATFINITE, __NV_E4M3);
                 const __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(
@@ -398,8 +403,10 @@ __device__ __forceinline__ void convert_block(const uint8_t *st, const float *mk
                           fmaf(x0.z, x_scale, m0.z), fmaf(x0.w, x_scale, m0.w),
                           fmaf(x1.x, x_scale, m1.x), fmaf(x1.y, x_scale, m1.y),
                           fmaf(x1.z, x_scale, m1.z), fmaf(x1.w, x_scale, m1.w)};
+            if (NORM) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) nrm = fmaf(y[e], y[e], nrm);
+                for (int e = 0; e < 8; ++e) nrm = fmaf(y[e], y[e], nrm);
+            }
             if (MODE == kBF16) {
                 uint32_t w[4];
 #pragma unroll
@@ -657,7 +664,7 @@ __device__ __forceinline__ void proj_tile(
             const float *mk = mcs + kb * C::BK;
             uint32_t wa[16];  // the row's A values of the stage (split: the hi part)
             uint32_t wl[16];  // split: the lo part
-            convert_block<MODE>(st, mk, r, x_scale, nrm, wa, wl);
+            convert_block<MODE, true>(st, mk, r, x_scale, nrm, wa, wl);
             // TMEM column c of a buffer holds the row's values of K offsets
             // c * (4 / element bytes) upward, lowest in the low bits
             tmem_st16(tq + ta_col<MODE>(s, 0), wa);
@@ -1065,7 +1072,7 @@ __device__ __forceinline__ void proj_persistent(const ProjBatch &batch, int *que
                 const float *mk = mcs + kb * C::BK;
                 uint32_t wa[16];  // the row's A values of the stage (split: the hi part)
                 uint32_t wl[16];  // split: the lo part
-                convert_block<MODE>(st, mk, r, x_scale, nrm, wa, wl);
+                convert_block<MODE, true>(st, mk, r, x_scale, nrm, wa, wl);
                 // TMEM column c of a buffer holds the row's values of K offsets
                 // c * (4 / element bytes) upward, lowest in the low bits
                 tmem_st16(tq + (DB ? kTADb + 16u * (uint32_t)s : ta_col<MODE>(s, 0)), wa);
@@ -1163,6 +1170,338 @@ __device__ __forceinline__ void proj_persistent(const ProjBatch &batch, int *que
                      "r"(C::TMEM)
                      : "memory");
     }
+}
+
+// ------------------------------------------------------------- CTA pairs
+// An arrival on the barrier of CTA `rank` of the pair at the same offset, MMAs
+// over both CTAs' rows (cta_group::2) and their commit to both CTAs.  What the
+// arrivals order passes through TMEM and the async proxy, under the tcgen05
+// fences: they need no cluster-wide release of the CTA's other memory (with
+// .release.cluster / .acquire.cluster the kernel took 6.07 instead of 4.06 ms
+// per 1M rows at d = 960).
+__device__ __forceinline__ void mbar_arrive_cl(uint64_t *bar, uint32_t rank) {
+    asm volatile(
+        "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
+        " mbarrier.arrive.shared::cluster.b64 _, [ra];\n}\n" ::"r"(smem_u32(bar)),
+        "r"(rank)
+        : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int MODE>
+__device__ __forceinline__ void umma2_ta_elect(uint32_t dtm, uint32_t atm, uint64_t b, uint32_t idesc,
+                                               uint32_t acc) {
+    if (MODE == kFP8) {
+        asm volatile(
+            "{\n .reg .pred e, p;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+            " @e tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtm),
+            "r"(atm), "l"(b), "r"(idesc), "r"(acc));
+    } else {
+        asm volatile(
+            "{\n .reg .pred e, p;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+            " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtm),
+            "r"(atm), "l"(b), "r"(idesc), "r"(acc));
+    }
+}
+__device__ __forceinline__ void umma2_commit_elect(uint64_t *bar) {
+    asm volatile(
+        "{\n .reg .pred e;\n .reg .b16 m;\n mov.b16 m, 3;\n elect.sync _|e, 0xffffffff;\n"
+        " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+        " [%0], m;\n}\n" ::"r"(smem_u32(bar))
+        : "memory");
+}
+
+// Two CTAs of a cluster on one tile of 256 rows x np columns (np a multiple of
+// 32): each copies and converts its own 128 rows of X (A in its TMEM, as
+// above) and copies half of the W tile, and the first CTA issues MMAs over
+// both (cta_group::2), for which each SM reads only its half of W from
+// shared memory.  Per K block of the split form the shared memory of an SM
+// then moves 62 KB (X in and out 32, W in 12, the MMAs' reads 18) instead of
+// 92 KB: 484 against 720 cycles at 128 B per clock, beside 577 cycles of
+// MMAs.  Clusters take the tiles c, c + clusters, ...; each accumulator is
+// drained by its own CTA before the next tile's first MMA.
+// The ring of copies (S slots: X and half a W tile) is deeper than the ring of
+// converted blocks in TMEM (NA buffers, as many as fit beside the
+// accumulators): a copy takes ~1,000 cycles, a conversion ~800.
+// Two groups of four converter warps, as in the other kernels (four groups:
+// 4.56 against 4.0 ms per 1M rows at d = 960).
+template <int MODE> struct PairCfg;
+template <> struct PairCfg<kSplit> {
+    static constexpr int S = 7, NA = 4, G = 2;
+    static constexpr uint32_t WB = 6144;  // half a W tile of at most 192 rows
+};
+template <int MODE> constexpr int pair_threads() { return 64 + 128 * PairCfg<MODE>::G; }
+template <int MODE> constexpr uint32_t pair_slot() {
+    return (uint32_t)Cfg<MODE>::XBOX * kXBox + (uint32_t)Cfg<MODE>::NB * PairCfg<MODE>::WB;
+}
+template <int MODE> constexpr uint32_t pair_smem(int dpad) {
+    return PairCfg<MODE>::S * pair_slot<MODE>() + 1024 + kBarArea + 512 + 4u * (uint32_t)dpad;
+}
+static_assert(pair_smem<kSplit>(6144) <= 227u * 1024u,
+              "the pair's slots exceed the dynamic shared memory of one CTA");
+static_assert(3u * 8u * 8u + 3u * 8u + 8u <= kBarArea, "barriers overflow their shared-memory area");
+
+template <int MODE>
+__device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGroup &P, int64_t total,
+                                          uint64_t wait_ns) {
+    using C = Cfg<MODE>;
+    constexpr int S = PairCfg<MODE>::S, NA = PairCfg<MODE>::NA, G = PairCfg<MODE>::G;
+    constexpr int kConv = 4 * G;  // converter warps
+    constexpr uint32_t SB = pair_slot<MODE>(), WB = PairCfg<MODE>::WB;
+    extern __shared__ uint8_t smem_raw[];
+    // the same offset in both CTAs: the dynamic shared memory starts alike
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *full = (uint64_t *)(smem + S * SB);
+    uint64_t *conv = full + S;   // first CTA: both CTAs' converters
+    uint64_t *empty = conv + S;
+    uint64_t *accf = empty + S;
+    uint64_t *acc_empty = accf + 1;      // first CTA: both CTAs' converters
+    uint64_t *mma_done = acc_empty + 1;
+    uint32_t *tmem_slot = (uint32_t *)(mma_done + 1);
+    volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    float *nrm_part = (float *)(smem + S * SB + kBarArea);   // 128 floats
+    float *mcs = (float *)(smem + S * SB + kBarArea + 512);  // nkb * BK floats
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int64_t c0 = blockIdx.x >> 1, cstep = gridDim.x >> 1;
+    const int nkb = P.nkb, np = P.np, npass = P.npass, dk = P.dk;
+    int *err = P.err;
+
+    for (int k = threadIdx.x; k < nkb * C::BK; k += (int)blockDim.x) mcs[k] = P.mcs_g[k];
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&conv[s], 8);  // one group of converters of each CTA
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(accf, 1);
+        mbar_init(acc_empty, 2 * kConv);
+        mbar_init(mma_done, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(C::TMEM)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // the other CTA's barriers are initialised
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)tmxp) : "memory");
+            const uint8_t *wt0 = P.wt0, *wt1 = P.wt1;
+            const uint32_t wb = (uint32_t)np * 32u;  // bytes of half a W tile
+            const uint32_t tx = (uint32_t)C::XBOX * kXBox + (uint32_t)C::NB * wb;
+            uint32_t it = 0;  // K blocks issued over all tiles
+            bool ok = true;
+            for (int64_t b = c0; b < total && ok; b += cstep) {
+                const int pass = (int)(b % npass);
+                const int row0 = (int)((b / npass * 2 + rank) * kBM);
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const int s = (int)(it % (uint32_t)S);
+                    const uint32_t ph = (it / (uint32_t)S) & 1u;
+                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, err, 1, wait_ns)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t *st = smem + s * SB;
+                    mbar_expect_tx(&full[s], tx);
+#pragma unroll
+                    for (int bx = 0; bx < C::XBOX; ++bx)
+                        tma_load_2d(st + bx * kXBox, tmxp, kb * C::BK + bx * 32, row0, &full[s]);
+                    uint8_t *bs = st + b_offset<MODE>();
+                    const int64_t wo = ((int64_t)pass * nkb + kb) * np * 64 + rank * wb;
+                    bulk_load(bs, wt0 + wo, wb, &full[s]);
+                    if (C::NB == 2) bulk_load(bs + WB, wt1 + wo, wb, &full[s]);
+                    if (kb + kPrefetch < nkb)
+#pragma unroll
+                        for (int bx = 0; bx < C::XBOX; ++bx)
+                            tma_prefetch_2d(tmxp, (kb + kPrefetch) * C::BK + bx * 32, row0);
+                }
+            }
+            // drain: the last loads of each stage must land before the CTA exits
+            for (uint32_t i = it > (uint32_t)S ? it - (uint32_t)S : 0u; i < it; ++i) {
+                const int s = (int)(i % (uint32_t)S);
+                const uint32_t ph = (i / (uint32_t)S) & 1u;
+                const uint64_t t0 = globaltimer();
+                while (!mbar_try(&full[s], ph) && globaltimer() - t0 < kWaitNs) {
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (rank == 0) {
+            // the whole warp runs the loop, one lane elected inside each
+            // instruction issues (see proj_persistent)
+            const uint32_t tmw = __reduce_or_sync(0xffffffffu, tmem);
+            const uint32_t idesc = (umma_idesc_base<MODE>() & ~(31u << 24)) |
+                                   (uint32_t)(2 * kBM >> 4) << 24 | ((uint32_t)(np >> 3) << 17);
+            const uint64_t d0 = umma_desc(smem_u32(smem) + b_offset<MODE>());
+            uint32_t sl = 0, ph = 0, ab = 0, t = 0;  // slot and its phase, A buffer, tile
+            bool ok = true;
+            for (int64_t b = c0; b < total && ok; b += cstep, ++t) {
+                if (t >= 1) {
+                    const bool r = mbar_wait(acc_empty, (t - 1u) & 1u, abort_flag, err, 2, wait_ns);
+                    if (!__all_sync(0xffffffffu, r)) break;
+                }
+                for (int kb = 0; kb < nkb; ++kb) {
+                    const bool r = mbar_wait(&conv[sl], ph, abort_flag, err, 2, wait_ns);
+                    if (!__all_sync(0xffffffffu, r)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t b0 = d0 + (uint64_t)(sl * (SB >> 4)), b1 = b0 + (WB >> 4);
+                    const uint32_t ahi = tmw + ta_col<MODE>((int)ab, 0), alo = tmw + ta_col<MODE>((int)ab, 1);
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk) {  // two 32-byte K steps per 64-byte row
+                        const uint64_t off = (uint64_t)(kk * 2);
+                        const uint32_t ka = 8u * (uint32_t)kk;
+                        umma2_ta_elect<MODE>(tmw, ahi + ka, b0 + off, idesc, (kb | kk) != 0);
+                        if (MODE == kSplit) {
+                            umma2_ta_elect<MODE>(tmw + kAcc2, ahi + ka, b1 + off, idesc, (kb | kk) != 0);
+                            umma2_ta_elect<MODE>(tmw + kAcc2, alo + ka, b0 + off, idesc, 1u);
+                        }
+                    }
+                    umma2_commit_elect(&empty[sl]);
+                    if (++sl == (uint32_t)S) {
+                        sl = 0;
+                        ph ^= 1u;
+                    }
+                    if (++ab == (uint32_t)NA) ab = 0;
+                }
+                umma2_commit_elect(accf);
+            }
+            // every MMA issued (see the end)
+            umma2_commit_elect(mma_done);
+        }
+        __syncwarp();
+    } else {
+        // ---- converters and epilogue, as in proj_persistent
+        const int q = warp & 3;
+        const int r = q * 32 + lane;
+        const int h = (warp - 2) >> 2;
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
+        const float x_scale = P.x_scale;
+        uint32_t base = 0, t = 0;
+        bool ok = true;
+        for (int64_t b = c0;; b += cstep, ++t) {
+            // the converter warps stop together (the end of the work, or a
+            // failed wait in any of them)
+            if (named_any(kBarStop, 32 * kConv, !ok || b >= total)) break;
+            const int pass = (int)(b % npass);
+            const int64_t row0 = (b / npass * 2 + rank) * kBM;
+            const int col0 = pass * np;
+            const bool row_ok = row0 + r < P.n;
+            float nrm = 0.f;
+            for (int kb = h; kb < nkb && ok; kb += G) {
+                const uint32_t it = base + (uint32_t)kb;
+                const int s = (int)(it % (uint32_t)S);
+                const uint32_t ph = (it / (uint32_t)S) & 1u;
+                int gotk = 0;
+                if (lane == 0)
+                    gotk = mbar_wait(&full[s], ph, abort_flag, err, 3, wait_ns) ? 1 : 0;
+                gotk = __shfl_sync(0xffffffffu, gotk, 0);
+                if (!gotk) {
+                    ok = false;
+                    break;
+                }
+                uint8_t *st = smem + s * SB;
+                const float *mk = mcs + kb * C::BK;
+                uint32_t wa[16], wl[16];
+                if (pass == 0) {  // uniform
+                    convert_block<MODE, true>(st, mk, r, x_scale, nrm, wa, wl);
+                } else {
+                    convert_block<MODE, false>(st, mk, r, x_scale, nrm, wa, wl);
+                }
+                // the A buffer is free once the MMAs of block it - NA are done
+                // (their slot's barrier can be no phase further: its next
+                // block comes after this one); waited for only now, so that
+                // the conversion runs ahead of the MMAs
+                if (it >= (uint32_t)NA) {
+                    const uint32_t old = it - (uint32_t)NA;
+                    if (lane == 0)
+                        gotk = mbar_wait(&empty[old % (uint32_t)S], (old / (uint32_t)S) & 1u, abort_flag,
+                                         err, 5, wait_ns)
+                                   ? 1
+                                   : 0;
+                    gotk = __shfl_sync(0xffffffffu, gotk, 0);
+                    if (!gotk) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                }
+                const int ab = (int)(it % (uint32_t)NA);
+                tmem_st16(tq + ta_col<MODE>(ab, 0), wa);
+                if (MODE == kSplit) tmem_st16(tq + ta_col<MODE>(ab, 1), wl);
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cl(&conv[s], 0);
+            }
+            static_assert(G == 2, "two partial sums of a row's norm, as in the other kernels");
+            if (pass == 0) {  // uniform
+                if (h == 1) nrm_part[r] = nrm;
+                named_sync(kBarNorm, 32 * kConv);
+            }
+            if (h == 0 && pass == 0 && row_ok && ok) {
+                const float tot = nrm + nrm_part[r];
+                if (P.norms) P.norms[(row0 + r) * P.nstride] = tot / (x_scale * x_scale);
+                if (!(tot < P.norm_limit)) atomicCAS(P.err, 0, kErrRange);
+            }
+            int ready = 0;
+            if (ok && lane == 0)
+                ready = mbar_wait(accf, t & 1u, abort_flag, err, 4, wait_ns) ? 1 : 0;
+            ready = __shfl_sync(0xffffffffu, ready, 0);
+            if (!ready) ok = false;
+            if (ready) {
+                tc_fence_after();
+                tile_epilogue<MODE>(tq, h, G, lane, r, row0, row_ok, np, col0, dk, P.col_scale, P.O,
+                                    P.ldo, P.il, P.vmax, P.segc);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cl(acc_empty, 0);
+            base += (uint32_t)nkb;
+        }
+        tc_fence_before();
+    }
+    __syncthreads();
+    // every MMA issued must be complete, and its commits delivered here, before
+    // TMEM and the barriers go (the first CTA commits this at its end whatever
+    // happened before)
+    if (warp == 1 && lane == 0) {
+        const uint64_t t0 = globaltimer();
+        while (!mbar_try(mma_done, 0) && globaltimer() - t0 < kWaitNs) {
+        }
+    }
+    __syncthreads();
+    // both CTAs are done with each other's barriers, W halves and TMEM
+    cluster_sync();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(C::TMEM)
+                     : "memory");
+    }
+}
+
+template <int MODE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<MODE>(), 1)
+k_proj_tc_pair(const __grid_constant__ ProjGroup P, int64_t total, uint64_t wait_ns) {
+    proj_pair<MODE>(&P.tmx, P, total, wait_ns);
 }
 
 // Persistent projection of a serving batch: one CTA per SM, each taking tiles
@@ -1577,6 +1916,38 @@ saq_status launch_grouped_mode(const ProjJob *jobs, int njobs, int *queue, cudaS
     return launch_persistent<MODE>(b, dpad_max, queue, db, s);
 }
 
+// One model's rows on the pair kernel: as many clusters of two CTAs as run at
+// once (an odd SM of its group has no partner), each with its share of the `total` tiles of 256
+// rows.
+template <int MODE>
+saq_status launch_pair(const ProjGroup &g, int64_t total, int dpad, uint64_t wait_ns, cudaStream_t s) {
+    if (total > 0x3FFFFFFF) return set_error(SAQ_ERR_UNSUPPORTED, "too many rows in one call");
+    const uint32_t sm = pair_smem<MODE>(dpad);
+    SAQ_CUDA_CHECK(cudaFuncSetAttribute(k_proj_tc_pair<MODE>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(sm_count() & ~1));
+    cfg.blockDim = dim3(pair_threads<MODE>());
+    cfg.dynamicSmemBytes = sm;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    SAQ_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, k_proj_tc_pair<MODE>, &cfg));
+    clusters = std::max(clusters, 1);
+    {
+        LaunchTimer lt_(kKindProject, s);
+        k_proj_tc_pair<MODE><<<(unsigned)(2 * std::min<int64_t>(total, clusters)), pair_threads<MODE>(),
+                               sm, s>>>(g, total, wait_ns);
+    }
+    note_launches();
+    SAQ_CUDA_CHECK(cudaGetLastError());
+    return SAQ_OK;
+}
+
 // One model's rows on the persistent kernel (db: the double-buffered one).
 // The work counter: none for at most a tile per SM, else `queue` (zero at
 // launch), or one of its own from the stream-ordered pool.
@@ -1595,6 +1966,17 @@ saq_status launch_persistent_single(const saq_model *m, const float *X, int64_t 
     if (st != SAQ_OK) return st;
     b.tile_start[0] = 0;
     b.tile_start[1] = rt * b.g[0].npass;
+    if constexpr (MODE == kSplit) {
+        // More than one tile per SM: pairs of SMs on tiles of 256 rows (see
+        // proj_pair; whole launches, pair against the single-SM kernel:
+        // 1,000,000 rows at d = 960 4.11 against 4.47 ms, 20,000 at 3072 738
+        // against 850 us, 100,000 at 1536 972 against 1,062 us, 40,000 at
+        // 128 20.8 against 20.3 us).  With fewer tiles, pairs would leave SMs
+        // idle; passes whose width is no multiple of 32 have no halves the
+        // MMA takes.
+        if (b.tile_start[1] > sm_count() && ex->np % 32 == 0)
+            return launch_pair<MODE>(b.g[0], (rt + 1) / 2 * ex->npass, m->tc.d_pad, b.wait_ns, s);
+    }
     if (b.tile_start[1] <= sm_count())
         return launch_persistent<MODE>(b, m->tc.d_pad, nullptr, db, s);
     if (queue) return launch_persistent<MODE>(b, m->tc.d_pad, queue, db, s);
