@@ -8,8 +8,8 @@
 // ballot finds the first that moves, its state is broadcast, and the lanes
 // after it try again.  Every decision is taken from the state the sequential
 // scan has at that coordinate, with the same operations, so the codes are the
-// same; the lane-per-vector kernel takes ~94 cycles a coordinate and round
-// when a warp has an SM to itself (448 coordinates: 143 us).
+// same; the lane-per-vector kernel takes ~65 cycles a coordinate and round
+// when a warp has an SM to itself (448 coordinates: 96 us).
 //
 // A block takes R rows of one kept segment (R = its warps).  The rows are
 // staged in shared memory (R + 1 floats per coordinate: conflict-free for
@@ -210,20 +210,21 @@ saq_status launch_caq_scan(const CaqJob *jobs, int njobs, cudaStream_t s, bool *
         coords += jobs[i].n * jobs[i].m->dk;
         for (const KeptSeg &k : jobs[i].m->kept) {
             maxlen = std::max(maxlen, (int)k.len);
-            chain = std::max(chain, (int)(k.bits == 1 ? k.len / 3 : k.len));
+            chain = std::max(chain, (int)(k.bits == 1 ? (k.len + 3) / 4 : k.len));
         }
     }
     if (used == 0 || scan_smem(maxlen, 8) > kScanSmemMax) return SAQ_OK;
     // 16 rows per block where their rows fit three blocks to an SM
     const bool r16 = scan_smem(maxlen, 16) <= 75 * 1024;
     // The lane-per-vector kernel takes at least its longest segment's chain of
-    // steps (0.42 us a coordinate at 6 rounds, a third of it at 1 bit, where
-    // the first round moves nothing); the scan takes 14 ns per 1,000
-    // coordinates, 25-30 with blocks of 8 rows.  Both cross, measured, at
-    // 14-20K rows of d = 960 (448-long, 4 b/dim: 13.4 M coordinates), 18K of
-    // d = 128 (64-long), 14K of d = 1536 (704-long), 4-5K of d = 3072 at 1
-    // b/dim and 17K at 8.
-    if (coords > (int64_t)(r16 ? 30000 : 15000) * chain) return SAQ_OK;
+    // steps (0.21-0.23 us a coordinate at 6 rounds, a quarter of it at 1 bit,
+    // where the first round moves nothing); the scan takes 12-13 ns per 1,000
+    // coordinates, 21-32 where one block fills an SM's shared memory.  Both
+    // cross, measured, at 6.2K rows of d = 960 (448-long, 4 b/dim; 99 us), 8.4K
+    // of d = 128 (64-long; 22 us), 7.6K of d = 1536 (704-long; 154 us), 1.95K of
+    // d = 3072 at 1 b/dim (98 us) and 7.0K at 8 (706 us).
+    const bool shared = r16 || scan_smem(maxlen, 8) <= 75 * 1024;
+    if (coords > (int64_t)(shared ? 15000 : 7500) * chain) return SAQ_OK;
     *ran = true;
     if (used == 1) {
         CaqBatch<1> b;
