@@ -26,17 +26,16 @@
 // into bit-planes, during the last round (or, for a warp whose lanes all stop
 // earlier, in a pass of its own).
 //
-// The kernel is bound by the instructions it issues (82% of the issue slots with
-// 16 warps per SM, ncu; the rows' DRAM traffic is at a third of its peak).  A
-// step took ~26 instructions, and at 32 warps per SM each round read the rows
-// from HBM anew.  Now a step is 16 (the update predicated instead of branched
-// around, codes turned into u two at a time, moves summed as floats), rows come
-// by asynchronous copies of 2 KB per warp, which need no registers, and 20 warps
-// per SM keep the issue slots filled while more of the rows they return to stay
-// in L2.  1,000,000 rows at d = 960, 4 b/dim 5.11 -> 4.28 ms; 100,000 at d =
-// 1536, 2 b/dim 716 -> 549 us; 65,537 at d = 3072, 1 b/dim 471 -> 344 us; a
-// 3,072-long segment at 8 bits of 20,011 rows, which waits for its own chain of
-// steps, 1,745 -> 854 us.
+// The kernel is bound by the instructions it issues (79% of the issue slots,
+// ncu; its DRAM traffic runs at 4.2 TB/s).  A step took ~26 instructions, and at
+// 32 warps per SM each round read the rows from HBM anew.  Now a step is 16 (the
+// update predicated instead of branched around, codes turned into u two at a
+// time, moves summed as floats), rows come by asynchronous copies of 2 KB per
+// warp, which need no registers, and 20 warps per SM keep the issue slots filled
+// while a part of the rows they return to stays in L2.  1,000,000 rows at d =
+// 960, 4 b/dim 5.11 -> 4.03 ms; 100,000 at d = 1536, 2 b/dim 716 -> 510 us;
+// 65,537 at d = 3072, 1 b/dim 471 -> 321 us; a 3,072-long segment at 8 bits of
+// 20,011 rows, which waits for its own chain of steps, 1,745 -> 729 us.
 #include <algorithm>
 #include <atomic>
 
@@ -237,30 +236,29 @@ template <int D, bool CODES> struct Ring {
 #pragma unroll 1
         for (int i = 0; i < D; ++i) issue(i * kSlot);
     }
-    // the rows of the batch at j0, complete in its slot (those past the
-    // segment's end are not to be used)
-    __device__ __forceinline__ void take(int j0, float (&x)[kU]) const {
-        if ((j0 & kU) == 0) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
-            __syncwarp();
-        }
-        const float *p = reinterpret_cast<const float *>(sm + slot + (j0 & kU) * 128) + lane;
+    // the next slot is complete
+    __device__ __forceinline__ void wait() const {
+        asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
+        __syncwarp();
+    }
+    // the rows of batch h of the slot (those past the segment's end are not to
+    // be used), and its codes
+    __device__ __forceinline__ void take(int h, float (&x)[kU]) const {
+        const float *p = reinterpret_cast<const float *>(sm + slot + h * (kU * 128)) + lane;
 #pragma unroll
         for (int k = 0; k < kU; ++k) x[k] = p[k * 32];
     }
-    __device__ __forceinline__ void take_codes(int j0, uint32_t (&w)[2]) const {
+    __device__ __forceinline__ void take_codes(int h, uint32_t (&w)[2]) const {
         const uint32_t *p =
-            reinterpret_cast<const uint32_t *>(sm + slot + kRows + (j0 & kU) * 32) + lane;
+            reinterpret_cast<const uint32_t *>(sm + slot + kRows + h * (kU * 32)) + lane;
         w[0] = p[0];
         w[1] = p[32];
     }
-    // after the last batch of a slot is taken: gives it to the copy D slots on
-    __device__ __forceinline__ void pass(int j0) {
-        if ((j0 & kU) || j0 + kU >= len) {
-            __syncwarp();
-            issue(slot);
-            slot = slot + kSlot < kBytes ? slot + kSlot : 0;
-        }
+    // the slot is taken: gives it to the copy D slots on
+    __device__ __forceinline__ void pass() {
+        __syncwarp();
+        issue(slot);
+        slot = slot + kSlot < kBytes ? slot + kSlot : 0;
     }
     // before the slots are used for anything else
     __device__ __forceinline__ void finish() const {
@@ -499,14 +497,18 @@ __device__ __forceinline__ void load_codes(const CS &cs, const typename CS::R &r
                                            int len, uint32_t (&w)[Fields<CS::kBits>::kWords]) {
     if constexpr (CS::kRingCodes) {
         if (n >= kU && len > kSlotCols * CS::kDepth) {
-            ring.take_codes(j0, w);
+            ring.take_codes((j0 / kU) & 1, w);
             return;
         }
     }
     cs.load(j0, w, n);
 }
 
-// One round of Algorithm 1 over the lane's segment.  With PACK_B = B > 0 the
+// One round of Algorithm 1 over the lane's segment, a slot of the ring at a time:
+// both batches are read before the first one's steps, so that the second's reads
+// and the next copy run beside them (a batch at a time: 4.28 ms per 1,000,000
+// rows at d = 960, 850 us for the 3,072-long segment of 20,011 rows; so: 4.03 and
+// 729).  With PACK_B = B > 0 the
 // round is the last one: a coordinate's code is final once its own step is
 // done, so the bit-planes (most significant first, 64-bit words) and the exact
 // |u|^2, which the function returns, are built as the round goes.
@@ -516,29 +518,42 @@ __device__ __forceinline__ int run_round(LaneState &L, typename CS::R &ring, con
                                          int words) {
     using F = Fields<CS::kBits>;
     const float cmaxf = (float)cmax, ucst = -(65536.f + cmaxf);
-    const int lenU = len & ~(kU - 1);  // coordinates in whole batches
+    const int lenU = len & ~(kSlotCols - 1);  // coordinates in whole slots
     Planes<PACK_B ? PACK_B : 1, CS::kBits> P;
     uint32_t any = 0u;
-    for (int j0 = 0; j0 < lenU; j0 += kU) {
-        float x[kU];
-        uint32_t w[F::kWords];
-        ring.take(j0, x);
-        load_codes(cs, ring, j0, kU, len, w);
-        ring.pass(j0);
-        const uint32_t ch = batch_steps<CS::kBits, true>(L, x, w, kU, cmaxf, ucst);
-        any |= ch;
-        if (PACK_B > 0) P.add(w, j0, kU, len, valid, cout, words);
-        else if (!CS::kWriteChanged || ch) cs.store(j0, w, kU);
+    for (int j0 = 0; j0 < lenU; j0 += kSlotCols) {
+        float x[2][kU];
+        uint32_t w[2][F::kWords];
+        ring.wait();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            ring.take(h, x[h]);
+            load_codes(cs, ring, j0 + h * kU, kU, len, w[h]);
+        }
+        ring.pass();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + h * kU;
+            const uint32_t ch = batch_steps<CS::kBits, true>(L, x[h], w[h], kU, cmaxf, ucst);
+            any |= ch;
+            if (PACK_B > 0) P.add(w[h], j, kU, len, valid, cout, words);
+            else if (!CS::kWriteChanged || ch) cs.store(j, w[h], kU);
+        }
     }
-    if (lenU < len) {  // the last, partial batch
-        float x[kU];
-        uint32_t w[F::kWords];
-        ring.take(lenU, x);
-        load_codes(cs, ring, lenU, len - lenU, len, w);
-        ring.pass(lenU);
-        any |= batch_steps<CS::kBits, false>(L, x, w, len - lenU, cmaxf, ucst);
-        if (PACK_B > 0) P.add(w, lenU, len - lenU, len, valid, cout, words);
-        else cs.store(lenU, w, len - lenU);
+    if (lenU < len) {  // the last, partial slot
+        ring.wait();
+#pragma unroll 1
+        for (int j = lenU; j < len; j += kU) {
+            const int n = min(kU, len - j);
+            float x[kU];
+            uint32_t w[F::kWords];
+            ring.take((j / kU) & 1, x);
+            load_codes(cs, ring, j, n, len, w);
+            any |= batch_steps<CS::kBits, false>(L, x, w, n, cmaxf, ucst);
+            if (PACK_B > 0) P.add(w, j, n, len, valid, cout, words);
+            else cs.store(j, w, n);
+        }
+        ring.pass();
     }
     moved = any != 0u;
     return PACK_B > 0 ? P.u2(len) : 0;
@@ -602,34 +617,44 @@ __device__ __forceinline__ void caq_segment(const CS &cs, typename CS::R ring, i
         sums(x[1], u1);
     };
     ring.start();
-    const int lenU = len & ~(kU - 1);  // coordinates in whole batches
-    for (int j0 = 0; j0 < lenU; j0 += kU) {
-        float x[kU], t[kU], cf[kU];
-        ring.take(j0, x);
-        ring.pass(j0);
+    const int lenU = len & ~(kSlotCols - 1);  // coordinates in whole slots
+    for (int j0 = 0; j0 < lenU; j0 += kSlotCols) {
+        float x[2][kU];
+        ring.wait();
+        ring.take(0, x[0]);
+        ring.take(1, x[1]);
+        ring.pass();
 #pragma unroll
-        for (int k = 0; k < kU; k += 2) init(&x[k], &t[k], &cf[k]);
-        uint32_t w[F::kWords];
-        F::pack(t, cf, w);
-        cs.store(j0, w, kU);
+        for (int h = 0; h < 2; ++h) {
+            float t[kU], cf[kU];
+#pragma unroll
+            for (int k = 0; k < kU; k += 2) init(&x[h][k], &t[k], &cf[k]);
+            uint32_t w[F::kWords];
+            F::pack(t, cf, w);
+            cs.store(j0 + h * kU, w, kU);
+        }
     }
     if (lenU < len) {
-        float x[kU], t[kU], cf[kU];
-        ring.take(lenU, x);
-        ring.pass(lenU);
+        ring.wait();
+#pragma unroll 1
+        for (int j = lenU; j < len; j += kU) {
+            float x[kU], t[kU], cf[kU];
+            ring.take((j / kU) & 1, x);
 #pragma unroll
-        for (int k = 0; k < kU; ++k) {
-            codes_of(x[k], x[k], t[k], t[k], cf[k], cf[k]);
-            if (lenU + k < len) {
-                sums(x[k], fmaf(2.f, cf[k], -cmaxf));
-            } else {
-                t[k] = 8388608.f;
-                cf[k] = 0.f;
+            for (int k = 0; k < kU; ++k) {
+                codes_of(x[k], x[k], t[k], t[k], cf[k], cf[k]);
+                if (j + k < len) {
+                    sums(x[k], fmaf(2.f, cf[k], -cmaxf));
+                } else {
+                    t[k] = 8388608.f;
+                    cf[k] = 0.f;
+                }
             }
+            uint32_t w[F::kWords];
+            F::pack(t, cf, w);
+            cs.store(j, w, min(kU, len - j));
         }
-        uint32_t w[F::kWords];
-        F::pack(t, cf, w);
-        cs.store(lenU, w, len - lenU);
+        ring.pass();
     }
     LaneState L{I, S, live ? I * I : __int_as_float(0x7f800000)};
     int Si = -1;  // |u|^2 of the final codes, exactly, once they are packed
@@ -731,7 +756,7 @@ __device__ __forceinline__ void caq1_warp(int64_t w, const float *__restrict__ O
 // All kept segments of a chunk in one launch.  Blocks of four warps, five of
 // them per SM at the d = 960 plan (44 KB each; 80 registers a thread, nothing
 // spilled): 4.28 ms per 1,000,000 rows, with blocks of eight (two per SM) 4.54,
-// of two 4.36.
+// of two 4.36, when the rows were taken a batch at a time (now 4.03).
 __global__ void __launch_bounds__(kWarps * 32, 5)
 k_caq1(const float *__restrict__ Oi, int64_t n, int dk, int nseg, const SegTable t, int rounds,
        uint8_t *__restrict__ cs, const float *__restrict__ vmax_arr,

@@ -8,8 +8,8 @@
 // ballot finds the first that moves, its state is broadcast, and the lanes
 // after it try again.  Every decision is taken from the state the sequential
 // scan has at that coordinate, with the same operations, so the codes are the
-// same; the lane-per-vector kernel takes ~65 cycles a coordinate and round
-// when a warp has an SM to itself (448 coordinates: 96 us).
+// same; the lane-per-vector kernel takes ~54 cycles a coordinate and round
+// when a warp has an SM to itself (448 coordinates: 82 us).
 //
 // A block takes R rows of one kept segment (R = its warps).  The rows are
 // staged in shared memory (R + 1 floats per coordinate: conflict-free for
@@ -217,14 +217,15 @@ saq_status launch_caq_scan(const CaqJob *jobs, int njobs, cudaStream_t s, bool *
     // 16 rows per block where their rows fit three blocks to an SM
     const bool r16 = scan_smem(maxlen, 16) <= 75 * 1024;
     // The lane-per-vector kernel takes at least its longest segment's chain of
-    // steps (0.21-0.23 us a coordinate at 6 rounds, a quarter of it at 1 bit,
-    // where the first round moves nothing); the scan takes 12-13 ns per 1,000
-    // coordinates, 21-32 where one block fills an SM's shared memory.  Both
-    // cross, measured, at 6.2K rows of d = 960 (448-long, 4 b/dim; 99 us), 8.4K
-    // of d = 128 (64-long; 22 us), 7.6K of d = 1536 (704-long; 154 us), 1.95K of
-    // d = 3072 at 1 b/dim (98 us) and 7.0K at 8 (706 us).
+    // steps (0.18 us a coordinate at 6 rounds, a quarter of it at 1 bit, where
+    // the first round moves nothing); the scan takes 12-16 ns per 1,000
+    // coordinates, 21-32 where one block fills an SM's shared memory.  Either
+    // side of the line, scan and lane-per-vector: d = 960 (448-long, 4 b/dim)
+    // 5,500 rows 87.6 us, 5,700 82.1; d = 128 (64-long) 5,900 18.0, 6,100 18.0;
+    // d = 1536 (704-long) 5,400 114, 5,600 125; d = 3072 at 1 b/dim 1,150 59,
+    // 1,190 79, at 8 b/dim 5,900 584, 6,100 555.
     const bool shared = r16 || scan_smem(maxlen, 8) <= 75 * 1024;
-    if (coords > (int64_t)(shared ? 15000 : 7500) * chain) return SAQ_OK;
+    if (coords > (int64_t)(shared ? 12000 : 6000) * chain) return SAQ_OK;
     *ran = true;
     if (used == 1) {
         CaqBatch<1> b;
