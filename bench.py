@@ -40,12 +40,12 @@ UNIT = "vectors/s"
 # a launch's traffic is proportional to its rows.  A figure is reported only while the
 # kernel's source file is the one that was captured (SHA-1 below).
 NCU_TRAFFIC = {
-    "projection": {"src": "k_tc.cu", "sha1": "957519d74ad2b945597249c6b3734e933f4f3071",
+    "projection": {"src": "k_tc.cu", "sha1": "07e142e51602bd811a34b18382be30015d87d53c",
                    "workload": "c2_d960", "precision": "fp32",
-                   "bytes_per_row": (258402304 + 211736064) / 65536},
-    "quantize_adjust_pack": {"src": "k_caq1.cu", "sha1": "ca5627b928766d09ea89518c720662654251fdcb",
+                   "bytes_per_row": (258268672 + 215917056) / 65536},
+    "quantize_adjust_pack": {"src": "k_caq1.cu", "sha1": "e0d5c197e0a71dfbc166d5b7a8a145f68b5d2a1f",
                              "workload": "c2_d960", "precision": "fp32",
-                             "bytes_per_row": (1558764544 + 35263744) / 65536},
+                             "bytes_per_row": (1173351680 + 25230336) / 65536},
 }
 
 
