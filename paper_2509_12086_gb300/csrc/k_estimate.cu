@@ -15,21 +15,33 @@
 // variance of <o_seg, q_seg> over the data:
 //   lb_t = |o_r - c|^2 + |q_r - c|^2 - 2 (sum_{s<t} est_s + m sum_{s>=t} sigma_s).
 //
-// <u_s, q_s> = 2 <c_s, q_s> - (2^b - 1) sum q_s.  <c_s, q_s> of 16 vectors and
-// 4 queries at a time is a matrix product on the tensor cores (mma.sync
-// m16n8k16, FP16 operands, FP32 accumulators).  A code's bits are its A
-// operand as they stand: read as a subnormal FP16 number they are c 2^-24, so
-// decoding is the bit-plane transposition, a shift and a mask.  Each query
-// coordinate is a pair of integers, hi + lo / 4096 with |hi| <= 2048 (23 bits
-// below the query's largest coordinate), in two columns of B.  Products and
-// sums are integers (times 2^-24), which FP32 holds exactly up to 2^24: the
-// tensor core's truncating accumulation loses nothing, the subtraction of
-// the code's mean is exact too, and the inner products are as good as an FP32
-// sum of the products (errors against 64 bits measured slightly below those
-// of the per-lane FP32 sums used before).
+// <c_s, q_s> of 16 vectors and 4 queries at a time is a matrix product on the
+// tensor cores (mma.sync m16n8k16, FP16 operands, FP32 accumulators).  A code's
+// bits are its A operand as they stand: read as a subnormal FP16 number they
+// are c 2^-24, so decoding is the bit-plane transposition, a shift and a mask.
+// Each query coordinate, times a power of two of its own (query, segment), is
+// a pair hi + lo / 4096 in two columns of B: hi an integer, lo the FP16 value
+// of what it leaves (at least 23 bits below the larger of hi and 2048).
+//
+// The tensor core truncates its sums, so those of hi, which carry the result's
+// leading bits, are kept exact: the accumulator starts at -2^(b-1) sum hi and
+// holds <c - 2^(b-1), hi> at the end, and while
+//     2^(b-1) sum |hi| <= 2^24
+// every partial sum is an integer (times 2^-24) that FP32 represents.  The
+// scale is the largest power of two for which that holds, whatever the
+// coordinates' signs and sizes are.  The sums run over a window of the segment:
+// all of it up to 4 bits, 128 2^(8-b) coordinates from 5 bits up, where one
+// window of a long segment would leave hi too few bits; windows are added up in
+// FP32.  <u, q> = 2 <c - 2^(b-1), hi> + sum hi + (2 <c, lo> - (2^b - 1) sum lo) / 4096.
+// Largest error over |u| |q| (512 vectors by 24 queries, 960 long at 8 bits, against
+// 64 bits; in brackets of sums of the products by FP32 lanes, and of queries
+// with one scale each whose <c, hi> were summed over the whole segment from 0):
+// Gaussian coordinates 1.8e-8 (2.0e-8, 3.0e-8), all of one sign 2.2e-8 (2.1e-8,
+// 4.1e-6), one of 1,000 among Gaussians 2.0e-8 (2.3e-8, 1.4e-7).
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cfloat>
 
 #include "saq_internal.h"
 
@@ -38,7 +50,8 @@ namespace saq {
 namespace {
 
 struct SegDesc {
-    int off, len, bits, words, fidx;
+    int off, len, bits, words, fidx;  // bits: those that the estimate reads
+    int step, window;                 // its first K step and window
     long long code_off;
 };
 constexpr int kMaxSeg = 64;
@@ -47,9 +60,8 @@ struct SegTable {
 };
 
 // ------------------------------------------------------------ the queries
-// out[q * dk + j] = <M_j, q_r - c> for the rows M_j of a dk x d matrix; with
-// qn2 also |q_r - c|^2 and, into qmax (zero before), the largest |out| of each
-// query (bits of a non-negative float order as integers).  A warp computes
+// out[q * dk + j] = <M_j, q_r - c> for the rows M_j of a dk x d matrix, and with
+// qn2 also |q_r - c|^2.  A warp computes
 // CPW columns for QB queries: its lanes split the d coordinates (the rows of
 // M are read once, coalesced, and each value meets QB centred queries in
 // shared memory), so that a single query spreads over dk warps (d = 960: 8.5
@@ -59,7 +71,7 @@ template <int QB, int CPW, bool V4>
 __global__ void __launch_bounds__(256)
 k_query_rot(const float *__restrict__ Q, int64_t nq, int d, const float *__restrict__ mean,
             const float *__restrict__ M, int dk, float *__restrict__ out,
-            float *__restrict__ qn2, unsigned *__restrict__ qmax) {
+            float *__restrict__ qn2) {
     static_assert(QB * CPW == 32 || QB * CPW == 1, "one result per lane, or one per warp");
     __shared__ __align__(16) float qs[QB][kRotK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -123,10 +135,7 @@ k_query_rot(const float *__restrict__ Q, int64_t nq, int d, const float *__restr
         float s = acc[0];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0 && j0 < dk) {
-            out[q0 * dk + j0] = s;
-            if (qmax) atomicMax(qmax + q0, __float_as_uint(fabsf(s)));
-        }
+        if (lane == 0 && j0 < dk) out[q0 * dk + j0] = s;
     } else {
         // 32 sums over 32 lanes: each exchange halves the values a lane holds,
         // and lane i ends with sum i (column i / QB, query i % QB)
@@ -141,14 +150,7 @@ k_query_rot(const float *__restrict__ Q, int64_t nq, int d, const float *__restr
         }
         const int j = j0 + lane / QB;
         const int64_t q = q0 + lane % QB;
-        const bool ok = j < dk && q < nq;
-        if (ok) out[q * dk + j] = acc[0];
-        if (qmax) {
-            unsigned mx = ok ? __float_as_uint(fabsf(acc[0])) : 0u;
-#pragma unroll
-            for (int off = QB; off < 32; off <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            if (lane < QB && q < nq) atomicMax(qmax + q, mx);
-        }
+        if (j < dk && q < nq) out[q * dk + j] = acc[0];
     }
 }
 
@@ -169,12 +171,34 @@ __global__ void k_query_sigma(const float *__restrict__ pc, int64_t nq, int dk, 
     if (lane == 0) sig[q * nk + s] = sqrtf(acc);
 }
 
-// The exponent that brings a query's largest coordinate into [1024, 2048)
-// (0 for an all-zero query or one that is not finite, whose estimates are
-// not finite either).
-__device__ __forceinline__ int query_exponent(unsigned mx) {
-    if (mx == 0u || mx >= 0x7F800000u) return 0;
-    return min(120, 10 - ilogbf(__uint_as_float(mx)));
+// Widths up to kNarrow bits take a segment as one window.
+constexpr int kNarrow = 4;
+// Pieces (of 128 coordinates, see step_coord) of a window at `bits` > kNarrow:
+// 2^(bits-1) times a window's coordinates is 16,384, which leaves hi a scale of
+// ~1,000 per standard deviation of a Gaussian window.
+__host__ __device__ constexpr int window_pieces(int bits) { return 1 << (8 - bits); }
+// Windows of a segment of `words` 64-bit words.
+constexpr int window_count(int bits, int words) {
+    return bits <= kNarrow ? 1 : ((words + 1) / 2 + window_pieces(bits) - 1) / window_pieces(bits);
+}
+// Bits that a segment's estimate reads.
+constexpr int used_bits(int prefix_bits, int bits) {
+    return prefix_bits > 0 && prefix_bits < bits ? prefix_bits : bits;
+}
+
+// The exponent of a (query, segment)'s scale, from the largest window sum l1 of
+// |q| and the largest |q|: 2^(b-1) sum |hi| <= 2^24 (rounding adds at most 1/2 to
+// each of a window's n coordinates, or 2^-11 of it above 2048) and |hi| <= 2^15.
+// 0 for an all-zero query or one that is not finite, whose estimates are not
+// finite either.
+__device__ __forceinline__ int scale_exponent(float l1, float mx, int bits, int n) {
+    constexpr float kSlack = 1.f - 0x1p-10f;
+    if (!(l1 <= FLT_MAX))  // NaN, an infinity, or finite values whose sum is not
+        return l1 == l1 && mx <= FLT_MAX ? -126 : 0;
+    if (l1 == 0.f) return 0;
+    const float b = fmaxf((float)(1 << (25 - bits)) - 0.5f * (float)n, 1.f) * kSlack;
+    const int e = min(ilogbf(b) - ilogbf(l1), 14 - ilogbf(mx));  // within one of the answer
+    return max(-126, min(100, e - (scalbnf(l1, e) > b || scalbnf(mx, e) > 32768.f * kSlack)));
 }
 
 // The coordinate (of a segment of `words` 64-bit words) that element i (0..3)
@@ -192,47 +216,145 @@ __device__ __forceinline__ int step_coord(int words, int step, int t, int i) {
     return at + ((words & 2) ? 128 : 0) + 16 * t + 4 * k + r + 8 * hi;
 }
 
-// B fragments of every pass: entry ((pass * steps + step) * NT + nt) * 32 +
-// lane holds the four FP16 values of column lane / 4 (query 4 (pass * NT +
-// nt) + column / 2, hi or lo part) for lane quad position lane % 4.  qsum
-// (zero before) takes the sum of each column over each segment.
+// B fragments of four queries (block x: column group pass * NT + nt) and one
+// segment (block y): entry ((pass * steps + step) * NT + nt) * 32 + lane holds
+// the four FP16 values of column lane / 4 (query 4 (pass * NT + nt) + column / 2,
+// hi or lo part) for lane quad position lane % 4.  Also, of each query, the
+// accumulators' start in every window, -2^(b-1) sum hi (times 2^-24),
+// wstart[((pass * windows + window) * NT + nt) * 4 + query], and per segment
+// qseg[((pass * segments + segment) * NT + nt) * 4 + query]: the inverse scale and
+// what completes <u, q>, sum hi and -(2^b - 1) sum lo / 4096.
+constexpr int kSplitPieces = 1024;  // pieces whose sums are held at a time
+constexpr int kSplitWindows = 64;
 __global__ void __launch_bounds__(256)
-k_query_split(const float *__restrict__ qrot, int64_t nq, int dk, int nk,
-              const __grid_constant__ SegTable t, int steps, int NT, int64_t total,
-              const unsigned *__restrict__ qmax, uint2 *__restrict__ bfrag,
-              int *__restrict__ qsum, int64_t cols) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const int lane = (int)(e & 31);
-    const int64_t f = e >> 5;
-    const int nt = (int)(f % NT);
-    const int gstep = (int)((f / NT) % steps);
-    const int64_t pass = f / NT / steps;
-    const int64_t q = 4 * (pass * NT + nt) + (lane >> 3);
-    const bool lo = (lane >> 2) & 1;
-    int s = 0, step = gstep;
-    while (s + 1 < nk && step >= 4 * t.s[s].words) step -= 4 * t.s[s++].words;
-    __half h[4];
-    int sum = 0;
+k_query_split(const float *__restrict__ qrot, int64_t nq, int dk,
+              const __grid_constant__ SegTable t, int steps, int NT, int windows,
+              uint2 *__restrict__ bfrag, float *__restrict__ wstart, float4 *__restrict__ qseg) {
+    __shared__ float piece[4][kSplitPieces];
+    __shared__ float part[kSplitWindows][8][8];
+    __shared__ float wmax[8], s_scale[4], s_inverse[4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t group = blockIdx.x, pass = group / NT, q0 = 4 * group;
+    const int nt = (int)(group % NT);
+    const int s = blockIdx.y;
+    const int len = t.s[s].len, words = t.s[s].words, bits = t.s[s].bits;
+    const float *src = qrot + q0 * dk + t.s[s].off;
+    // ---- the scales: warp w takes the pieces of query w % 4 in turn
+    const int pieces = (words + 1) / 2, full = words >> 2;
+    const int P = bits <= kNarrow ? pieces : window_pieces(bits), nwin = (pieces + P - 1) / P;
+    {
+        const int b = warp & 3;
+        const float *p = src + (int64_t)b * dk;
+        const bool live = q0 + b < nq;
+        float mx = 0.f, l1 = 0.f;  // of lane 0 .. 31's windows
+        for (int p0 = 0; p0 < pieces; p0 += kSplitPieces) {
+            const int pn = min(kSplitPieces, pieces - p0);
+#pragma unroll 4
+            for (int i = warp >> 2; i < pn; i += 2) {
+                const int pi = p0 + i;
+                float a = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int c = step_coord(t.s[s].words, step, lane & 3, i);
-        float v = 0.f;
-        if (q < nq && c < t.s[s].len) {
-            const float y = scalbnf(qrot[q * dk + t.s[s].off + c], query_exponent(qmax[q]));
-            const float r = rintf(y);
-            v = lo ? rintf((y - r) * 4096.f) : r;
+                for (int j = 0; j < 4; ++j) {
+                    const int c = pi < 2 * full
+                                      ? (4 * (pi >> 1) + j) * 64 + (pi & 1) * 32 + lane
+                                      : 256 * full + (pi - 2 * full) * 128 + 32 * j + lane;
+                    const float v = live && c < len ? fabsf(__ldg(p + c)) : 0.f;
+                    a += v;
+                    mx = fmaxf(mx, v);
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+                if (lane == 0) piece[b][i] = a;
+            }
+            __syncthreads();
+            if (warp < 4) {
+                if (nwin == 1) {
+                    for (int i = lane; i < pn; i += 32) l1 += piece[b][i];
+                } else {  // P divides kSplitPieces
+                    for (int w = lane; w * P < pn; w += 32) {
+                        float a = 0.f;
+                        for (int i = w * P; i < min(pn, w * P + P); ++i) a += piece[b][i];
+                        l1 = a > l1 || a != a ? a : l1;  // a NaN stays
+                    }
+                }
+            }
+            __syncthreads();
         }
-        h[i] = __float2half_rn(v);
-        sum += (int)v;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float o = __shfl_xor_sync(0xffffffffu, l1, off);
+            l1 = nwin == 1 ? l1 + o : o > l1 || o != o ? o : l1;
+        }
+        if (lane == 0) wmax[warp] = mx;
+        __syncthreads();
+        if (warp < 4 && lane == 0) {
+            const int e = scale_exponent(l1, fmaxf(wmax[b], wmax[b + 4]), bits, min(len, 128 * P));
+            s_scale[b] = scalbnf(1.f, e);
+            s_inverse[b] = scalbnf(1.f, -e);
+        }
+        __syncthreads();
     }
-    uint2 o;
-    o.x = (uint32_t)__half_as_ushort(h[0]) | (uint32_t)__half_as_ushort(h[1]) << 16;
-    o.y = (uint32_t)__half_as_ushort(h[2]) | (uint32_t)__half_as_ushort(h[3]) << 16;
-    bfrag[e] = o;
-    sum += __shfl_xor_sync(0xffffffffu, sum, 1);  // total is a multiple of 32: whole warps
-    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-    if ((lane & 3) == 0) atomicAdd(qsum + s * cols + 8 * (pass * NT + nt) + (lane >> 2), sum);
+    // ---- the columns, a K step per warp, and their sums by windows: G warps to
+    // a window
+    int G = 8;
+    while (G > 1 && nwin * G > 8) G >>= 1;
+    const int wg = warp / G, wi = warp % G;
+    const int b = lane >> 3;
+    const bool lo = (lane >> 2) & 1, live = q0 + b < nq;
+    const float scale = s_scale[b];
+    const float *p = src + (int64_t)b * dk;
+    uint2 *out = bfrag + ((pass * steps + t.s[s].step) * NT + nt) * 32 + lane;
+    float total = 0.f;  // of column threadIdx.x < 8 over the segment
+    for (int v0 = 0; v0 < nwin; v0 += kSplitWindows) {
+        const int vn = min(kSplitWindows, nwin - v0);
+        for (int v = wg; v < vn; v += 8 / G) {
+            const int first = 8 * P * (v0 + v), last = min(4 * words, first + 8 * P);
+            float sum = 0.f;
+#pragma unroll 4
+            for (int step = first + wi; step < last; step += G) {
+                __half h[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int c = step_coord(words, step, lane & 3, i);
+                    float x = 0.f;
+                    if (live && c < len) {
+                        const float y = __ldg(p + c) * scale;
+                        const float r = fabsf(y) < 2048.f ? rintf(y) : __half2float(__float2half_rn(y));
+                        x = lo ? (y - r) * 4096.f : r;
+                    }
+                    h[i] = __float2half_rn(x);
+                    sum += __half2float(h[i]);
+                }
+                uint2 o;
+                o.x = (uint32_t)__half_as_ushort(h[0]) | (uint32_t)__half_as_ushort(h[1]) << 16;
+                o.y = (uint32_t)__half_as_ushort(h[2]) | (uint32_t)__half_as_ushort(h[3]) << 16;
+                out[(int64_t)step * NT * 32] = o;
+            }
+            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+            if ((lane & 3) == 0) part[v][wi][lane >> 2] = sum;
+        }
+        __syncthreads();
+        const float start = -(float)(1 << (bits - 1)) * 0x1p-24f;
+        for (int e = threadIdx.x; e < 8 * vn; e += 256) {
+            const int v = e >> 3, c = e & 7;
+            float sum = 0.f;  // hi: integers below 2^24, in any order exact
+            for (int w = 0; w < G; ++w) sum += part[v][w][c];
+            part[v][0][c] = sum;
+            if (!(c & 1)) wstart[((pass * windows + t.s[s].window + v0 + v) * NT + nt) * 4 + (c >> 1)] = start * sum;
+        }
+        __syncthreads();
+        if (threadIdx.x < 8)
+            for (int v = 0; v < vn; ++v) total += part[v][0][threadIdx.x];
+        __syncthreads();
+    }
+    if (warp == 0) {
+        const float lo_sum = __shfl_down_sync(0xffffffffu, total, 1);
+        if (lane < 8 && !(lane & 1))
+            qseg[((pass * gridDim.y + s) * NT + nt) * 4 + (lane >> 1)] = make_float4(
+                s_inverse[lane >> 1], total, -(float)((1 << bits) - 1) * 0x1p-12f * lo_sum, 0.f);
+    }
 }
 
 // ------------------------------------------------------------ the vectors
@@ -307,13 +429,13 @@ struct EstArgs {
     const float *factors;
     int nf;
     int64_t n;
-    int nk, prefix_bits;
+    int nk;
     const uint2 *bfrag;
     int steps;
     const float *qn2;
-    const unsigned *qmax;
-    const int *qsum;  // per segment and B column: the sum of the column over the segment
-    int64_t cols;     // B columns of all passes
+    const float *wstart;  // of a pass, per window and query (see k_query_split)
+    const float4 *qseg;   // of a pass, per segment and query
+    int windows;          // of all segments
     int64_t nq;
     const float *qsig;  // staged: sigma of (query, segment)
     float m_conf;
@@ -353,14 +475,66 @@ template <bool SM, class T> __device__ __forceinline__ T load_rec(const void *p)
     else return __ldg(static_cast<const T *>(p));
 }
 
+// A window's accumulators at its start (ws: the lane's query's of the first B
+// tile), and what it adds to <u, q> at its end: 2 <c - 2^(b-1), hi> and
+// 2 <c, lo> / 4096, from sums that are times 2^-24.
+template <bool BS, int NT, int MT>
+__device__ __forceinline__ void open_window(const float *__restrict__ ws, float (&acc)[MT][NT][4]) {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        const float h = load_rec<BS, float>(ws + 4 * nt);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            acc[mt][nt][0] = acc[mt][nt][2] = h;
+            acc[mt][nt][1] = acc[mt][nt][3] = 0.f;
+        }
+    }
+}
+template <int NT, int MT>
+__device__ __forceinline__ void close_window(const float (&acc)[MT][NT][4], float (&tot)[MT][NT][2]) {
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                tot[mt][nt][h] = fmaf(fmaf(acc[mt][nt][2 * h + 1], 0x1p-12f, acc[mt][nt][2 * h]), 0x1p25f,
+                                      tot[mt][nt][h]);
+}
+
 // The products of one segment of `bits` bits (its first planes; at most NP)
-// for the warp's rows (row pointers at the segment's codes).  S2 += sum c^2 and
-// S1 += sum c over the lane's coordinates.
-template <int NP, int NT, int MT, bool SM>
+// for the warp's rows (row pointers at the segment's codes).  tot = <u, q>
+// (scaled), S2 += sum c^2 and S1 += sum c over the lane's coordinates.  ws and
+// qs: wstart and qseg of the segment at the lane's query of the first B tile (4 NT
+// of them a window or segment).
+template <int NP, int NT, int MT, bool SM, bool BS>
 __device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], int bits, int words,
                                             int len, int t, const uint2 *__restrict__ b,
-                                            float (&acc)[MT][NT][4],
+                                            const float *__restrict__ ws,
+                                            const float4 *__restrict__ qs,
+                                            float (&tot)[MT][NT][2],
                                             uint32_t (&S2)[MT][2], uint32_t (&S1)[MT][2]) {
+    float acc[MT][NT][4];
+    open_window<BS, NT, MT>(ws, acc);
+    // sum hi is small beside <u, q> from 5 bits up
+    if constexpr (NP > kNarrow)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            const float4 c = load_rec<BS, float4>(qs + 4 * nt);
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) tot[mt][nt][0] = tot[mt][nt][1] = c.y + c.z;
+        }
+    // the window ends before piece i (one window up to kNarrow bits, where
+    // NP is 4)
+    const int P = window_pieces(bits);
+    auto window_ends = [&](int i) {
+        if constexpr (NP > kNarrow) {
+            if (i == 0 || (i & (P - 1)) != 0) return;  // uniform
+            close_window<NT, MT>(acc, tot);
+            ws += 4 * NT;
+            open_window<BS, NT, MT>(ws, acc);
+        }
+    };
     const bool partial = (len & 63) != 0;  // bits past the end are to read as zero
     // sum of the codes of one lane's plane words
     auto code_sum = [](const uint32_t (&w)[NP]) {
@@ -416,6 +590,7 @@ __device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], i
                 S2[mt][h] = cd[mt][h].sum2(S2[mt][h]);
             }
         if (i + 1 < pieces) fetch(i + 1);
+        window_ends(i);
         run_steps<NP, NT, MT, 8>(cd, b, acc);
         b += 8 * NT * 32;
     }
@@ -439,7 +614,23 @@ __device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], i
                 cd[mt][h].split(w);
                 S2[mt][h] = cd[mt][h].sum2(S2[mt][h]);
             }
+        window_ends(pieces);
         run_steps<NP, NT, MT, 4>(cd, b, acc);
+    }
+    if constexpr (NP > kNarrow) {
+        close_window<NT, MT>(acc, tot);
+    } else {
+        // an exact <u, hi> (at one bit it is small beside its parts), then lo's
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            const float4 c = load_rec<BS, float4>(qs + 4 * nt);
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    tot[mt][nt][h] = fmaf(acc[mt][nt][2 * h], 0x1p25f, c.y) +
+                                     fmaf(acc[mt][nt][2 * h + 1], 0x1p13f, c.z);
+        }
     }
 }
 
@@ -476,6 +667,16 @@ __device__ __forceinline__ void stage_tile(const EstArgs &A, int64_t r0, int row
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+// Shared memory of a pass's wstart and qseg.
+__host__ __device__ constexpr size_t table_bytes(int windows, int segments, int NT) {
+    return (size_t)(windows + 4 * segments) * 4 * NT * sizeof(float);
+}
+
+// Warps of a block of the staged form: with 24 (80 registers a thread) up to
+// four B tiles spill, 10 queries x 100K staged bounds at 8 b/dim 140 us, with 20
+// (96) 131.
+__host__ __device__ constexpr int staged_warps(int NT) { return NT <= 4 ? 20 : 12; }
+
 // A warp takes tiles of 16 MT vectors; the block's NT B columns (4 NT queries
 // of pass blockIdx.y) stay in shared memory (BS) for all of its tiles.
 // SM: the tile's code records and factors are copied to the warp's own buffer
@@ -483,27 +684,30 @@ __device__ __forceinline__ void stage_tile(const EstArgs &A, int64_t r0, int row
 // done), so that the loads of the decode take 30 cycles instead of an L2 or
 // HBM round trip at the start of every segment; the other warps of the SM
 // cover the copy.
-// Bound by the instructions of the decode (77% of the issue slots, 68% of the
-// integer pipe; HBM 20%, tensor pipe 10% at one query): 1 query x 1M records
-// of 480 B 4,350 -> 271 us, 100 x 100K 22,600 -> 224 us (the tensor pipe 42%),
-// against a warp per (query, vector) that decoded a bit per plane and lane.
+// Bound by the instructions of the decode: 1 query x 1M records of 480 B 4,350 ->
+// 279 us, 100 x 100K 22,600 -> 231 us, against a warp per (query, vector) that
+// decoded a bit per plane and lane.
 // Measured on the way: decode to FP16 integers by two more FP16 operations
 // per pair 405 us, |u|^2 from two more products per step (their diagonals)
 // 360 us, records read from global memory by every lane 390 us.
 template <int NT, int MT, bool BS, bool STAGED, bool SM>
-__global__ void __launch_bounds__(SM ? (NT <= 4 ? 768 : 384) : 256, 1)
+__global__ void __launch_bounds__(SM ? 32 * staged_warps(NT) : 256, 1)
 k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstride) {
     static_assert(!SM || MT == 1, "a staged tile holds 16 records");
     extern __shared__ __align__(16) uint2 bsm[];
-    __shared__ float s_qn2[4 * NT], s_qsc[4 * NT];
+    __shared__ float s_qn2[4 * NT];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int64_t q0 = (int64_t)blockIdx.y * 4 * NT;
     const uint2 *bg = A.bfrag + (int64_t)blockIdx.y * A.steps * NT * 32;
     const int64_t tiles = (A.n + 16 * MT - 1) / (16 * MT), tstep = (int64_t)gridDim.x * warps;
     int64_t tile = (int64_t)blockIdx.x * warps + warp;
+    // the pass's wstart and qseg, beside B where that is shared
+    const float *wstart = A.wstart + (int64_t)blockIdx.y * A.windows * (4 * NT);
+    const float4 *qseg = A.qseg + (int64_t)blockIdx.y * A.nk * (4 * NT);
+    float4 *tabs = reinterpret_cast<float4 *>(bsm + (BS ? A.steps * NT * 32 : 0));
     // the warp's buffer: 16 records, then their factors
-    uint8_t *buf = reinterpret_cast<uint8_t *>(bsm + (BS ? A.steps * NT * 32 : 0)) +
+    uint8_t *buf = reinterpret_cast<uint8_t *>(tabs) + (BS ? table_bytes(A.windows, A.nk, NT) : 0) +
                    (SM ? warp * (16 * sstride + ((64 * A.nf + 15) & ~15)) : 0);
     float *fbuf = reinterpret_cast<float *>(buf + 16 * sstride);
     if (SM && tile < tiles)
@@ -511,10 +715,17 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
     if constexpr (BS)
         for (int e = threadIdx.x; e < A.steps * NT * 16; e += blockDim.x)
             reinterpret_cast<uint4 *>(bsm)[e] = __ldg(reinterpret_cast<const uint4 *>(bg) + e);
+    if constexpr (BS) {
+        const int nw = A.windows * (4 * NT), ns = A.nk * (4 * NT);
+        float *ws = reinterpret_cast<float *>(tabs + ns);
+        for (int e = threadIdx.x; e < ns; e += blockDim.x) tabs[e] = __ldg(qseg + e);
+        for (int e = threadIdx.x; e < nw; e += blockDim.x) ws[e] = __ldg(wstart + e);
+        qseg = tabs;
+        wstart = ws;
+    }
     for (int e = threadIdx.x; e < 4 * NT; e += blockDim.x) {
         const int64_t q = q0 + e;
         s_qn2[e] = q < A.nq ? A.qn2[q] : 0.f;
-        s_qsc[e] = q < A.nq ? scalbnf(1.f, -query_exponent(A.qmax[q])) : 0.f;
     }
     __syncthreads();
     const uint2 *b0 = (BS ? bsm : bg) + lane;
@@ -558,7 +769,7 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
                         const int64_t q = q0 + 4 * nt + t;
                         if (q >= A.nq) continue;
                         const float base = f0 + s_qn2[4 * nt + t];
-                        const float e = est[mt][nt][h] * s_qsc[4 * nt + t];
+                        const float e = est[mt][nt][h];
                         if constexpr (STAGED) {
                             float rest = 0.f;  // m * sum_{s >= stage} sigma_s
                             for (int s = stage; s < A.nk; ++s) rest += __ldg(A.qsig + q * A.nk + s);
@@ -571,12 +782,11 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
                 }
         };
         if constexpr (STAGED) store(0);
-        int step0 = 0;
         for (int s = 0; s < A.nk; ++s) {
             const SegDesc &sg = tab.s[s];
-            const int bits = A.prefix_bits > 0 ? min(A.prefix_bits, sg.bits) : sg.bits;
+            const int bits = sg.bits;
             const uint8_t *rp[MT][2];
-            float acc[MT][NT][4];
+            float tot[MT][NT][2];
             uint32_t S2[MT][2], S1[MT][2];
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
@@ -584,24 +794,27 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
                 rp[mt][1] = rec[mt][1] + sg.code_off;
                 S2[mt][0] = S2[mt][1] = 0u;
                 S1[mt][0] = S1[mt][1] = 0u;
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
             }
             // the two factors of one of the lane quad's rows in each of its lanes
             const float *fv = fac[0][0];
 #pragma unroll
             for (int i = 1; i < 2 * MT; ++i)
                 if (t % (2 * MT) == i) fv = fac[i >> 1][i & 1];
-            const float nrm = load_rec<SM, float>(fv + sg.fidx);
-            const float cs = load_rec<SM, float>(fv + sg.fidx + 1);
-            const uint2 *b = b0 + step0 * NT * 32;
-            if (bits <= 4)  // uniform
-                run_segment<4, NT, MT, SM>(rp, bits, sg.words, sg.len, t, b, acc, S2, S1);
+            float nrm, cosine;
+            auto factors = [&] {
+                nrm = load_rec<SM, float>(fv + sg.fidx);
+                cosine = load_rec<SM, float>(fv + sg.fidx + 1);
+            };
+            // (before the products, unless the registers run short)
+            if constexpr (NT > 1) factors();
+            const uint2 *b = b0 + sg.step * NT * 32;
+            const float *ws = wstart + sg.window * (4 * NT) + t;
+            const float4 *qs = qseg + s * (4 * NT) + t;
+            if (bits <= kNarrow)  // uniform
+                run_segment<4, NT, MT, SM, BS>(rp, bits, sg.words, sg.len, t, b, ws, qs, tot, S2, S1);
             else
-                run_segment<8, NT, MT, SM>(rp, bits, sg.words, sg.len, t, b, acc, S2, S1);
-            step0 += 4 * sg.words;
+                run_segment<8, NT, MT, SM, BS>(rp, bits, sg.words, sg.len, t, b, ws, qs, tot, S2, S1);
+            if constexpr (NT == 1) factors();
             // |u|^2 = 4 (sum c^2 - cmax sum c) + len cmax^2, the sums spread
             // over the quad; lane t forms the scale of row t % (2 MT)
             const int cmax = (1 << bits) - 1;
@@ -626,26 +839,19 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
             const float S = sg.len > 65536
                                 ? (float)(4ll * c2 + (long long)sg.len * (cmax * cmax))
                                 : (float)(4u * (uint32_t)c2 + (uint32_t)sg.len * (uint32_t)(cmax * cmax));
-            const float vs = nrm > 0.f ? nrm / (sqrtf(S) * cs) : 0.f;
-            const float fc = -(float)cmax;
-            const int *qs = A.qsum + (int64_t)s * A.cols + (int64_t)blockIdx.y * 8 * NT + 2 * t;
+            const float vs = nrm > 0.f ? nrm / (sqrtf(S) * cosine) : 0.f;
             float vsr[MT][2];
 #pragma unroll
             for (int i = 0; i < 2 * MT; ++i)
                 vsr[i >> 1][i & 1] = __shfl_sync(0xffffffffu, vs, (g << 2) | i);
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
-                const int2 sum = __ldg(reinterpret_cast<const int2 *>(qs + 8 * nt));
-                const float sh = (float)sum.x, sl = (float)sum.y;
+                const float inv = load_rec<BS, float>(qs + 4 * nt);
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        // <u, hi> and <u, lo>: 2 <c, .> - cmax sum
-                        const float hi = fmaf(fc, sh, acc[mt][nt][2 * h] * 0x1p25f);
-                        const float lo = fmaf(fc, sl, acc[mt][nt][2 * h + 1] * 0x1p25f);
-                        est[mt][nt][h] = fmaf(fmaf(lo, 1.f / 4096.f, hi), vsr[mt][h], est[mt][nt][h]);
-                    }
+                    for (int h = 0; h < 2; ++h)
+                        est[mt][nt][h] = fmaf(tot[mt][nt][h] * inv, vsr[mt][h], est[mt][nt][h]);
             }
             if constexpr (STAGED) store(s + 1);
         }
@@ -660,11 +866,15 @@ k_estimate_mma(const EstArgs A, const __grid_constant__ SegTable tab, int sstrid
     }
 }
 
-SegTable seg_table(const saq_model *m) {
+SegTable seg_table(const saq_model *m, int prefix_bits) {
     SegTable t{};
+    int step = 0, window = 0;
     for (size_t i = 0; i < m->kept.size(); ++i) {
         const KeptSeg &k = m->kept[i];
-        t.s[i] = SegDesc{k.off, k.len, k.bits, k.words, k.fidx, (long long)k.code_off};
+        const int bits = used_bits(prefix_bits, k.bits);
+        t.s[i] = SegDesc{k.off, k.len, bits, k.words, k.fidx, step, window, (long long)k.code_off};
+        step += 4 * k.words;
+        window += window_count(bits, k.words);
     }
     return t;
 }
@@ -674,6 +884,13 @@ int total_steps(const saq_model *m) {
     int steps = 0;
     for (const KeptSeg &k : m->kept) steps += 4 * k.words;
     return steps;
+}
+
+// Windows over all kept segments.
+int total_windows(const saq_model *m, int prefix_bits) {
+    int n = 0;
+    for (const KeptSeg &k : m->kept) n += window_count(used_bits(prefix_bits, k.bits), k.words);
+    return n;
 }
 
 constexpr size_t kEstSmemMax = 224 * 1024;  // dynamic shared memory of a block
@@ -694,8 +911,11 @@ struct EstPlan {
     int64_t passes = 1;
     bool bs = true;  // B in shared memory (else read through the caches)
     int warps = 0;   // staged form: warps per block (0: the form without staging)
-    int64_t cols() const { return passes * NT * 8; }
 };
+// Bytes of a block's B columns and their tables.
+size_t column_bytes(const saq_model *m, int NT) {
+    return (size_t)total_steps(m) * NT * 256 + table_bytes(total_windows(m, 0), (int)m->kept.size(), NT);
+}
 // 4 NT queries per pass: the fewest passes whose B columns fit in shared
 // memory, then the smallest form that still does them in that many.  Records
 // are staged when the buffers of at least eight warps fit beside B.
@@ -708,7 +928,7 @@ EstPlan est_plan(const saq_model *m, int64_t nq) {
     const auto choose = [&](size_t beside) {
         int most = 0;
         for (int f : forms)
-            if ((size_t)p.steps * f * 256 + beside <= kEstSmemMax) most = f;
+            if (column_bytes(m, f) + beside <= kEstSmemMax) most = f;
         if (!most) return false;
         const int64_t need = (nts + (nts + most - 1) / most - 1) / ((nts + most - 1) / most);
         for (int f : forms)
@@ -720,8 +940,8 @@ EstPlan est_plan(const saq_model *m, int64_t nq) {
         return true;
     };
     if (choose(8 * wb)) {
-        const int fit = (int)((kEstSmemMax - (size_t)p.steps * p.NT * 256) / wb);
-        p.warps = std::min(p.NT <= 4 ? 24 : 12, fit);
+        const int fit = (int)((kEstSmemMax - column_bytes(m, p.NT)) / wb);
+        p.warps = std::min(staged_warps(p.NT), fit);
     } else if (!choose(0)) {
         p.bs = false;
         p.NT = 1;
@@ -732,10 +952,10 @@ EstPlan est_plan(const saq_model *m, int64_t nq) {
 
 template <int NT, int MT, bool BS, bool STAGED, bool SM>
 saq_status launch_form(const EstArgs &a, const SegTable &t, const EstPlan &p, int sstride,
-                       size_t wb, cudaStream_t s) {
+                       size_t cb, size_t wb, cudaStream_t s) {
     const auto kernel = k_estimate_mma<NT, MT, BS, STAGED, SM>;
     const int warps = SM ? p.warps : 8;
-    const size_t smem = (BS ? (size_t)a.steps * NT * 256 : 0) + (SM ? warps * wb : 0);
+    const size_t smem = (BS ? cb : 0) + (SM ? warps * wb : 0);
     int dev = 0, sms = 0, per_sm = 0;
     SAQ_CUDA_CHECK(cudaGetDevice(&dev));
     SAQ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -754,8 +974,8 @@ saq_status launch_form(const EstArgs &a, const SegTable &t, const EstPlan &p, in
         EstArgs b = a;
         b.bfrag += p0 * a.steps * NT * 32;
         b.qn2 += p0 * 4 * NT;
-        b.qmax += p0 * 4 * NT;
-        b.qsum += p0 * 8 * NT;
+        b.wstart += p0 * a.windows * 4 * NT;
+        b.qseg += p0 * a.nk * 4 * NT;
         if (STAGED) b.qsig += p0 * 4 * NT * a.nk;
         b.nq -= p0 * 4 * NT;
         b.out += p0 * 4 * NT * a.n * (STAGED ? a.nk + 1 : 1);
@@ -774,25 +994,25 @@ template <bool STAGED>
 saq_status launch_forms(const saq_model *m, const EstArgs &a, const SegTable &t, const EstPlan &p,
                         cudaStream_t s) {
     const int ss = staged_stride(m);
-    const size_t wb = staged_bytes(m);
-    if (!p.bs) return launch_form<1, 1, false, STAGED, false>(a, t, p, ss, wb, s);
+    const size_t cb = column_bytes(m, p.NT), wb = staged_bytes(m);
+    if (!p.bs) return launch_form<1, 1, false, STAGED, false>(a, t, p, ss, cb, wb, s);
     if (p.warps > 0) {
         switch (p.NT) {
-            case 1: return launch_form<1, 1, true, STAGED, true>(a, t, p, ss, wb, s);
-            case 4: return launch_form<4, 1, true, STAGED, true>(a, t, p, ss, wb, s);
-            default: return launch_form<8, 1, true, STAGED, true>(a, t, p, ss, wb, s);
+            case 1: return launch_form<1, 1, true, STAGED, true>(a, t, p, ss, cb, wb, s);
+            case 4: return launch_form<4, 1, true, STAGED, true>(a, t, p, ss, cb, wb, s);
+            default: return launch_form<8, 1, true, STAGED, true>(a, t, p, ss, cb, wb, s);
         }
     }
     switch (p.NT) {
-        case 1: return launch_form<1, 1, true, STAGED, false>(a, t, p, ss, wb, s);
-        case 4: return launch_form<4, 1, true, STAGED, false>(a, t, p, ss, wb, s);
-        default: return launch_form<8, 2, true, STAGED, false>(a, t, p, ss, wb, s);
+        case 1: return launch_form<1, 1, true, STAGED, false>(a, t, p, ss, cb, wb, s);
+        case 4: return launch_form<4, 1, true, STAGED, false>(a, t, p, ss, cb, wb, s);
+        default: return launch_form<8, 2, true, STAGED, false>(a, t, p, ss, cb, wb, s);
     }
 }
 
-// out = (Q - c) M^T (nq x dk) for a dk x d matrix, with max |out| per query.
+// out = (Q - c) M^T (nq x dk) for a dk x d matrix.
 saq_status launch_query_rot(const saq_model *m, const float *Q, int64_t nq, const float *M,
-                            float *out, float *qn2, unsigned *qmax, cudaStream_t s) {
+                            float *out, float *qn2, cudaStream_t s) {
     // a few queries: one column per warp, so that the rows of M spread over
     // the chip; more: eight queries share each row read
     const bool one = nq <= 2;
@@ -805,12 +1025,11 @@ saq_status launch_query_rot(const saq_model *m, const float *Q, int64_t nq, cons
         const float *Qp = Q + q0 * m->d;
         float *op = out + q0 * m->dk;
         float *np = qn2 ? qn2 + q0 : nullptr;
-        unsigned *mp = qmax ? qmax + q0 : nullptr;
         LaunchTimer lt_(kKindProject, s);
-        if (one && v4) k_query_rot<1, 1, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
-        else if (one) k_query_rot<1, 1, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
-        else if (v4) k_query_rot<8, 4, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
-        else k_query_rot<8, 4, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np, mp);
+        if (one && v4) k_query_rot<1, 1, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np);
+        else if (one) k_query_rot<1, 1, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np);
+        else if (v4) k_query_rot<8, 4, true><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np);
+        else k_query_rot<8, 4, false><<<grid, 256, 0, s>>>(Qp, n, m->d, m->d_mean, M, m->dk, op, np);
         note_launches();
     }
     SAQ_CUDA_CHECK(cudaGetLastError());
@@ -819,14 +1038,13 @@ saq_status launch_query_rot(const saq_model *m, const float *Q, int64_t nq, cons
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch: rotated queries, |q - c|^2, max |q_rot| and the column sums (both
-// zeroed before use), B fragments and, for the staged bounds, the basis values and sigma of (query, segment).
+// Scratch: rotated queries, |q - c|^2, wstart and qseg, B fragments and, for the staged bounds, the basis values
+// and sigma of (query, segment).
 struct EstScratch {
-    float *qrot, *qn2, *pc, *qsig;
-    unsigned *qmax;
-    int *qsum;
+    float *qrot, *qn2, *wstart, *pc, *qsig;
+    float4 *qseg;
     uint2 *bfrag;
-    size_t bytes, zero_bytes;
+    size_t bytes;
 };
 EstScratch est_scratch(const saq_model *m, int64_t nq, const EstPlan &p, bool staged, void *base) {
     EstScratch r{};
@@ -839,10 +1057,10 @@ EstScratch est_scratch(const saq_model *m, int64_t nq, const EstPlan &p, bool st
     const size_t dk = (size_t)std::max(1, m->dk), q = (size_t)nq;
     r.qrot = (float *)take(4 * q * dk);
     r.qn2 = (float *)take(4 * q);
-    const size_t at0 = at;
-    r.qmax = (unsigned *)take(4 * q);
-    r.qsum = (int *)take(4 * (size_t)p.cols() * std::max<size_t>(1, m->kept.size()));
-    r.zero_bytes = at - at0;
+    // (a prefix has no more windows)
+    const size_t queries = (size_t)p.passes * p.NT * 4;
+    r.wstart = (float *)take(4 * queries * (size_t)total_windows(m, 0));
+    r.qseg = (float4 *)take(16 * queries * m->kept.size());
     r.bfrag = (uint2 *)take((size_t)p.passes * p.steps * p.NT * 256);
     if (staged) {
         r.pc = (float *)take(4 * q * dk);
@@ -863,25 +1081,24 @@ saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float
                            float m_conf, void *scratch, float *out, cudaStream_t s) {
     const int nk = (int)m->kept.size();
     if (nk > kMaxSeg) return set_error(SAQ_ERR_UNSUPPORTED, "more than %d kept segments", kMaxSeg);
-    const SegTable t = seg_table(m);
+    const SegTable t = seg_table(m, prefix_bits);
     const EstPlan p = est_plan(m, nq);
     const EstScratch w = est_scratch(m, nq, p, staged, scratch);
-    SAQ_CUDA_CHECK(cudaMemsetAsync(w.qmax, 0, w.zero_bytes, s));
+    const int windows = total_windows(m, prefix_bits);
     if (nk == 0) {
         saq_status st = launch_rownorm2(m, Q, nq, w.qn2, 1, s);
         if (st != SAQ_OK) return st;
     } else {
-        saq_status st = launch_query_rot(m, Q, nq, m->d_W, w.qrot, w.qn2, w.qmax, s);
+        saq_status st = launch_query_rot(m, Q, nq, m->d_W, w.qrot, w.qn2, s);
         if (st != SAQ_OK) return st;
-        const int64_t total = p.passes * p.steps * p.NT * 32;
         {
             LaunchTimer lt_(kKindOther, s);
-            k_query_split<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-                w.qrot, nq, m->dk, nk, t, p.steps, p.NT, total, w.qmax, w.bfrag, w.qsum, p.cols());
+            k_query_split<<<dim3((unsigned)(p.passes * p.NT), (unsigned)nk), 256, 0, s>>>(
+                w.qrot, nq, m->dk, t, p.steps, p.NT, windows, w.bfrag, w.wstart, w.qseg);
         }
         note_launches();
         if (staged) {
-            st = launch_query_rot(m, Q, nq, m->d_B, w.pc, nullptr, nullptr, s);
+            st = launch_query_rot(m, Q, nq, m->d_B, w.pc, nullptr, s);
             if (st != SAQ_OK) return st;
             {
                 LaunchTimer lt_(kKindOther, s);
@@ -898,13 +1115,12 @@ saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float
     a.nf = m->nf;
     a.n = n;
     a.nk = nk;
-    a.prefix_bits = prefix_bits;
     a.bfrag = w.bfrag;
     a.steps = p.steps;
     a.qn2 = w.qn2;
-    a.qmax = w.qmax;
-    a.qsum = w.qsum;
-    a.cols = p.cols();
+    a.wstart = w.wstart;
+    a.qseg = w.qseg;
+    a.windows = windows;
     a.nq = nq;
     a.qsig = w.qsig;
     a.m_conf = m_conf;
