@@ -44,8 +44,8 @@
 //           a third of the MMAs, and the epilogue adds the two in FP32;
 //   kBF16   one BF16 product;
 //   kFP8    one E4M3 product (kind::f8f6f4), per-segment scales on W.
-// Large FP32 batches run on pairs of SMs, two CTAs to a tile of 256 rows (see
-// proj_pair); the rest is as above.
+// Large FP32 batches of more than 288 dimensions run on pairs of SMs, two CTAs
+// to a tile of 256 rows (see proj_pair); the rest is as above.
 // All waits are bounded (about 2 s); a timed-out wait raises an error flag,
 // every role leaves its loop, in-flight copies and MMAs are drained, TMEM is
 // freed and the kernel returns.
@@ -1967,14 +1967,19 @@ saq_status launch_persistent_single(const saq_model *m, const float *X, int64_t 
     b.tile_start[0] = 0;
     b.tile_start[1] = rt * b.g[0].npass;
     if constexpr (MODE == kSplit) {
-        // More than one tile per SM: pairs of SMs on tiles of 256 rows (see
-        // proj_pair; whole launches, pair against the single-SM kernel:
-        // 1,000,000 rows at d = 960 4.11 against 4.47 ms, 20,000 at 3072 738
-        // against 850 us, 100,000 at 1536 972 against 1,062 us, 40,000 at
-        // 128 20.8 against 20.3 us).  With fewer tiles, pairs would leave SMs
-        // idle; passes whose width is no multiple of 32 have no halves the
+        // More than one tile per SM and at least kPairBlocks K blocks: pairs
+        // of SMs on tiles of 256 rows (see proj_pair; whole launches, pair
+        // against the single-SM kernel: 1,000,000 rows at d = 960 4.11 against
+        // 4.47 ms, 20,000 at 3072 738 against 850 us, 100,000 at 1536 972
+        // against 1,062 us).  With fewer tiles, pairs would leave SMs idle; a
+        // pair's tile has a longer start and end to a shorter K loop (100,000
+        // rows at d = 128 38.9 against 36.9 us, at 256 79.3 against 78.3; means
+        // over 20,000-600,000 rows and kept widths from 32 up: d = 128 1.05 of
+        // the single-SM kernel's time, 256 1.02, 288-352 1.00, 512 0.99, 960
+        // 0.93); passes whose width is no multiple of 32 have no halves the
         // MMA takes.
-        if (b.tile_start[1] > sm_count() && ex->np % 32 == 0)
+        constexpr int kPairBlocks = 10;
+        if (b.tile_start[1] > sm_count() && b.g[0].nkb >= kPairBlocks && ex->np % 32 == 0)
             return launch_pair<MODE>(b.g[0], (rt + 1) / 2 * ex->npass, m->tc.d_pad, b.wait_ns, s);
     }
     if (b.tile_start[1] <= sm_count())
