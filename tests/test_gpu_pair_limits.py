@@ -40,3 +40,61 @@ def test_pairs_equal_single_tiles_at_the_line(d, dk, bits, tiles, extra):
         assert torch.equal(o, O[a:b]) and torch.equal(nr, norms[a:b]), a
         assert torch.equal(c, codes[a:b]) and torch.equal(f, factors[a:b]), a
     m.check_device()
+
+
+# ---- failures, as in test_gpu_failure.py, where the pair kernel runs
+N_TILES = 40  # beyond the SMs
+
+
+@pytest.fixture(scope="module")
+def batch():
+    m = _model(320, 320, 4, mean=0.0, rounds=2)
+    n = (_sms() + N_TILES) * 128 - 27
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.randn(n, 320, generator=g, device="cuda")
+    codes, factors = m.encode(X)
+    m.check_device()
+    return m, X, codes.clone(), factors.clone()
+
+
+def _encode_equals(m, X, codes, factors):
+    c, f = m.encode(X)
+    m.check_device()
+    assert torch.equal(c, codes) and torch.equal(f, factors)
+
+
+def test_wait_timeout_is_reported_and_the_next_encode_is_correct(batch):
+    m, X, codes, factors = batch
+    P.saq_set_wait_limit(1)
+    try:
+        for _ in range(3):
+            m.encode(X)
+            with pytest.raises(P.SaqError, match="timed out"):
+                m.check_device()
+        with pytest.raises(P.SaqError, match="timed out"):
+            m.encode_host(X.cpu().pin_memory())
+        m.project(X)
+        with pytest.raises(P.SaqError, match="timed out"):
+            m.check_device()
+    finally:
+        P.saq_set_wait_limit(0)
+    m.check_device()  # the flag was cleared by the reports
+    _encode_equals(m, X, codes, factors)
+
+
+# a row of the first CTA's half of a tile, of the second's, of the last, ragged tile
+@pytest.mark.parametrize("row", [5, 128 + 77, -1])
+@pytest.mark.parametrize("bad", ["large", "nan", "inf"])
+def test_bad_rows_are_reported(batch, row, bad):
+    m, X, codes, factors = batch
+    Y = X.clone()
+    if bad == "large":
+        Y[row] *= 3e4  # beyond the FP16 split's range
+    else:
+        Y[row, 319] = float(bad)
+    m.encode(Y)
+    with pytest.raises(P.SaqError, match="out of range"):
+        m.check_device()
+    m.check_device()
+    Y[row] = X[row]
+    _encode_equals(m, Y, codes, factors)
