@@ -65,7 +65,12 @@ struct SegTable {
 // CPW columns for QB queries: its lanes split the d coordinates (the rows of
 // M are read once, coalesced, and each value meets QB centred queries in
 // shared memory), so that a single query spreads over dk warps (d = 960: 8.5
-// us; on the 128 x 128 tiles of the row projection, eight blocks, 207 us).
+// us; on the 128 x 128 tiles of the row projection, eight blocks, 207 us).  Only
+// the coordinates there are get staged (with 1,024 whatever d is: 16,000 queries
+// at d = 128 79 -> 47 us, 8,000 at 1536 1,609 -> 1,264, 8,000 at 960 622 -> 611).
+// The row projection's tiles, whose sums run over all coordinates in one lane,
+// are as fast at 16,000 queries of 128 coordinates (44 us) and faster beyond
+// (64,000: 111 against 214).
 constexpr int kRotK = 1024;  // coordinates of the queries staged at a time
 template <int QB, int CPW, bool V4>
 __global__ void __launch_bounds__(256)
@@ -88,10 +93,11 @@ k_query_rot(const float *__restrict__ Q, int64_t nq, int d, const float *__restr
     for (int k0 = 0; k0 < d; k0 += kRotK) {
         const int kn = min(kRotK, d - k0);
         if (k0) __syncthreads();
-        for (int e = threadIdx.x; e < QB * kRotK; e += 256) {
-            const int b = e / kRotK, k = e % kRotK;
-            qs[b][k] = (k < kn && q0 + b < nq) ? Q[(q0 + b) * d + k0 + k] - mean[k0 + k] : 0.f;
-        }
+        constexpr int kTeam = 256 / QB;  // threads to a query
+        const int b = threadIdx.x / kTeam;
+#pragma unroll 8
+        for (int k = threadIdx.x % kTeam; k < kn; k += kTeam)
+            qs[b][k] = q0 + b < nq ? Q[(q0 + b) * d + k0 + k] - mean[k0 + k] : 0.f;
         __syncthreads();
         if (norm)
             for (int k = lane; k < kn; k += 32) n2 = fmaf(qs[warp][k], qs[warp][k], n2);
