@@ -1189,20 +1189,12 @@ __device__ __forceinline__ void mbar_arrive_cl(uint64_t *bar, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-template <int MODE>
 __device__ __forceinline__ void umma2_ta_elect(uint32_t dtm, uint32_t atm, uint64_t b, uint32_t idesc,
                                                uint32_t acc) {
-    if (MODE == kFP8) {
-        asm volatile(
-            "{\n .reg .pred e, p;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
-            " @e tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtm),
-            "r"(atm), "l"(b), "r"(idesc), "r"(acc));
-    } else {
-        asm volatile(
-            "{\n .reg .pred e, p;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
-            " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtm),
-            "r"(atm), "l"(b), "r"(idesc), "r"(acc));
-    }
+    asm volatile(
+        "{\n .reg .pred e, p;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtm),
+        "r"(atm), "l"(b), "r"(idesc), "r"(acc));
 }
 __device__ __forceinline__ void umma2_commit_elect(uint64_t *bar) {
     asm volatile(
@@ -1226,29 +1218,23 @@ __device__ __forceinline__ void umma2_commit_elect(uint64_t *bar) {
 // accumulators): a copy takes ~1,000 cycles, a conversion ~800.
 // Two groups of four converter warps, as in the other kernels (four groups:
 // 4.56 against 4.0 ms per 1M rows at d = 960).
-template <int MODE> struct PairCfg;
-template <> struct PairCfg<kSplit> {
-    static constexpr int S = 7, NA = 4, G = 2;
-    static constexpr uint32_t WB = 6144;  // half a W tile of at most 192 rows
-};
-template <int MODE> constexpr int pair_threads() { return 64 + 128 * PairCfg<MODE>::G; }
-template <int MODE> constexpr uint32_t pair_slot() {
-    return (uint32_t)Cfg<MODE>::XBOX * kXBox + (uint32_t)Cfg<MODE>::NB * PairCfg<MODE>::WB;
+constexpr int kPairS = 7, kPairNA = 4, kPairG = 2;
+constexpr uint32_t kPairWB = 6144;  // half a W tile of at most 192 rows
+constexpr int kPairThreads = 64 + 128 * kPairG;
+constexpr uint32_t kPairSlot = (uint32_t)Cfg<kSplit>::XBOX * kXBox + 2u * kPairWB;
+constexpr uint32_t pair_smem(int dpad) {
+    return kPairS * kPairSlot + 1024 + kBarArea + 512 + 4u * (uint32_t)dpad;
 }
-template <int MODE> constexpr uint32_t pair_smem(int dpad) {
-    return PairCfg<MODE>::S * pair_slot<MODE>() + 1024 + kBarArea + 512 + 4u * (uint32_t)dpad;
-}
-static_assert(pair_smem<kSplit>(6144) <= 227u * 1024u,
+static_assert(pair_smem(6144) <= 227u * 1024u,
               "the pair's slots exceed the dynamic shared memory of one CTA");
 static_assert(3u * 8u * 8u + 3u * 8u + 8u <= kBarArea, "barriers overflow their shared-memory area");
 
-template <int MODE>
 __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGroup &P, int64_t total,
                                           uint64_t wait_ns) {
-    using C = Cfg<MODE>;
-    constexpr int S = PairCfg<MODE>::S, NA = PairCfg<MODE>::NA, G = PairCfg<MODE>::G;
+    using C = Cfg<kSplit>;
+    constexpr int S = kPairS, NA = kPairNA, G = kPairG;
     constexpr int kConv = 4 * G;  // converter warps
-    constexpr uint32_t SB = pair_slot<MODE>(), WB = PairCfg<MODE>::WB;
+    constexpr uint32_t SB = kPairSlot, WB = kPairWB;
     extern __shared__ uint8_t smem_raw[];
     // the same offset in both CTAs: the dynamic shared memory starts alike
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1301,7 +1287,7 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)tmxp) : "memory");
             const uint8_t *wt0 = P.wt0, *wt1 = P.wt1;
             const uint32_t wb = (uint32_t)np * 32u;  // bytes of half a W tile
-            const uint32_t tx = (uint32_t)C::XBOX * kXBox + (uint32_t)C::NB * wb;
+            const uint32_t tx = (uint32_t)C::XBOX * kXBox + 2u * wb;
             uint32_t it = 0;  // K blocks issued over all tiles
             bool ok = true;
             for (int64_t b = c0; b < total && ok; b += cstep) {
@@ -1319,10 +1305,10 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
 #pragma unroll
                     for (int bx = 0; bx < C::XBOX; ++bx)
                         tma_load_2d(st + bx * kXBox, tmxp, kb * C::BK + bx * 32, row0, &full[s]);
-                    uint8_t *bs = st + b_offset<MODE>();
+                    uint8_t *bs = st + b_offset<kSplit>();
                     const int64_t wo = ((int64_t)pass * nkb + kb) * np * 64 + rank * wb;
                     bulk_load(bs, wt0 + wo, wb, &full[s]);
-                    if (C::NB == 2) bulk_load(bs + WB, wt1 + wo, wb, &full[s]);
+                    bulk_load(bs + WB, wt1 + wo, wb, &full[s]);
                     if (kb + kPrefetch < nkb)
 #pragma unroll
                         for (int bx = 0; bx < C::XBOX; ++bx)
@@ -1344,9 +1330,9 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
             // the whole warp runs the loop, one lane elected inside each
             // instruction issues (see proj_persistent)
             const uint32_t tmw = __reduce_or_sync(0xffffffffu, tmem);
-            const uint32_t idesc = (umma_idesc_base<MODE>() & ~(31u << 24)) |
+            const uint32_t idesc = (umma_idesc_base<kSplit>() & ~(31u << 24)) |
                                    (uint32_t)(2 * kBM >> 4) << 24 | ((uint32_t)(np >> 3) << 17);
-            const uint64_t d0 = umma_desc(smem_u32(smem) + b_offset<MODE>());
+            const uint64_t d0 = umma_desc(smem_u32(smem) + b_offset<kSplit>());
             uint32_t sl = 0, ph = 0, ab = 0, t = 0;  // slot and its phase, A buffer, tile
             bool ok = true;
             for (int64_t b = c0; b < total && ok; b += cstep, ++t) {
@@ -1362,16 +1348,14 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
                     }
                     tc_fence_after();
                     const uint64_t b0 = d0 + (uint64_t)(sl * (SB >> 4)), b1 = b0 + (WB >> 4);
-                    const uint32_t ahi = tmw + ta_col<MODE>((int)ab, 0), alo = tmw + ta_col<MODE>((int)ab, 1);
+                    const uint32_t ahi = tmw + ta_col<kSplit>((int)ab, 0), alo = tmw + ta_col<kSplit>((int)ab, 1);
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {  // two 32-byte K steps per 64-byte row
                         const uint64_t off = (uint64_t)(kk * 2);
                         const uint32_t ka = 8u * (uint32_t)kk;
-                        umma2_ta_elect<MODE>(tmw, ahi + ka, b0 + off, idesc, (kb | kk) != 0);
-                        if (MODE == kSplit) {
-                            umma2_ta_elect<MODE>(tmw + kAcc2, ahi + ka, b1 + off, idesc, (kb | kk) != 0);
-                            umma2_ta_elect<MODE>(tmw + kAcc2, alo + ka, b0 + off, idesc, 1u);
-                        }
+                        umma2_ta_elect(tmw, ahi + ka, b0 + off, idesc, (kb | kk) != 0);
+                        umma2_ta_elect(tmw + kAcc2, ahi + ka, b1 + off, idesc, (kb | kk) != 0);
+                        umma2_ta_elect(tmw + kAcc2, alo + ka, b0 + off, idesc, 1u);
                     }
                     umma2_commit_elect(&empty[sl]);
                     if (++sl == (uint32_t)S) {
@@ -1420,9 +1404,9 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
                 const float *mk = mcs + kb * C::BK;
                 uint32_t wa[16], wl[16];
                 if (pass == 0) {  // uniform
-                    convert_block<MODE, true>(st, mk, r, x_scale, nrm, wa, wl);
+                    convert_block<kSplit, true>(st, mk, r, x_scale, nrm, wa, wl);
                 } else {
-                    convert_block<MODE, false>(st, mk, r, x_scale, nrm, wa, wl);
+                    convert_block<kSplit, false>(st, mk, r, x_scale, nrm, wa, wl);
                 }
                 // the A buffer is free once the MMAs of block it - NA are done
                 // (their slot's barrier can be no phase further: its next
@@ -1443,8 +1427,8 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
                     tc_fence_after();
                 }
                 const int ab = (int)(it % (uint32_t)NA);
-                tmem_st16(tq + ta_col<MODE>(ab, 0), wa);
-                if (MODE == kSplit) tmem_st16(tq + ta_col<MODE>(ab, 1), wl);
+                tmem_st16(tq + ta_col<kSplit>(ab, 0), wa);
+                tmem_st16(tq + ta_col<kSplit>(ab, 1), wl);
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
@@ -1467,7 +1451,7 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
             if (!ready) ok = false;
             if (ready) {
                 tc_fence_after();
-                tile_epilogue<MODE>(tq, h, G, lane, r, row0, row_ok, np, col0, dk, P.col_scale, P.O,
+                tile_epilogue<kSplit>(tq, h, G, lane, r, row0, row_ok, np, col0, dk, P.col_scale, P.O,
                                     P.ldo, P.il, P.vmax, P.segc);
             }
             tc_fence_before();
@@ -1498,10 +1482,9 @@ __device__ __forceinline__ void proj_pair(const CUtensorMap *tmxp, const ProjGro
     }
 }
 
-template <int MODE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<MODE>(), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 k_proj_tc_pair(const __grid_constant__ ProjGroup P, int64_t total, uint64_t wait_ns) {
-    proj_pair<MODE>(&P.tmx, P, total, wait_ns);
+    proj_pair(&P.tmx, P, total, wait_ns);
 }
 
 // Persistent projection of a serving batch: one CTA per SM, each taking tiles
@@ -1919,11 +1902,10 @@ saq_status launch_grouped_mode(const ProjJob *jobs, int njobs, int *queue, cudaS
 // One model's rows on the pair kernel: as many clusters of two CTAs as run at
 // once (an odd SM of its group has no partner), each with its share of the `total` tiles of 256
 // rows.
-template <int MODE>
 saq_status launch_pair(const ProjGroup &g, int64_t total, int dpad, uint64_t wait_ns, cudaStream_t s) {
     if (total > 0x3FFFFFFF) return set_error(SAQ_ERR_UNSUPPORTED, "too many rows in one call");
-    const uint32_t sm = pair_smem<MODE>(dpad);
-    SAQ_CUDA_CHECK(cudaFuncSetAttribute(k_proj_tc_pair<MODE>,
+    const uint32_t sm = pair_smem(dpad);
+    SAQ_CUDA_CHECK(cudaFuncSetAttribute(k_proj_tc_pair,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1931,16 +1913,16 @@ saq_status launch_pair(const ProjGroup &g, int64_t total, int dpad, uint64_t wai
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sm_count() & ~1));
-    cfg.blockDim = dim3(pair_threads<MODE>());
+    cfg.blockDim = dim3(kPairThreads);
     cfg.dynamicSmemBytes = sm;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int clusters = 0;
-    SAQ_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, k_proj_tc_pair<MODE>, &cfg));
+    SAQ_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, k_proj_tc_pair, &cfg));
     clusters = std::max(clusters, 1);
     {
         LaunchTimer lt_(kKindProject, s);
-        k_proj_tc_pair<MODE><<<(unsigned)(2 * std::min<int64_t>(total, clusters)), pair_threads<MODE>(),
+        k_proj_tc_pair<<<(unsigned)(2 * std::min<int64_t>(total, clusters)), kPairThreads,
                                sm, s>>>(g, total, wait_ns);
     }
     note_launches();
@@ -1980,7 +1962,7 @@ saq_status launch_persistent_single(const saq_model *m, const float *X, int64_t 
         // MMA takes.
         constexpr int kPairBlocks = 10;
         if (b.tile_start[1] > sm_count() && b.g[0].nkb >= kPairBlocks && ex->np % 32 == 0)
-            return launch_pair<MODE>(b.g[0], (rt + 1) / 2 * ex->npass, m->tc.d_pad, b.wait_ns, s);
+            return launch_pair(b.g[0], (rt + 1) / 2 * ex->npass, m->tc.d_pad, b.wait_ns, s);
     }
     if (b.tile_start[1] <= sm_count())
         return launch_persistent<MODE>(b, m->tc.d_pad, nullptr, db, s);
