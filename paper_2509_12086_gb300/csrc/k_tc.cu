@@ -1174,11 +1174,23 @@ __device__ __forceinline__ void proj_persistent(const ProjBatch &batch, int *que
 
 // ------------------------------------------------------------- CTA pairs
 // An arrival on the barrier of CTA `rank` of the pair at the same offset, MMAs
-// over both CTAs' rows (cta_group::2) and their commit to both CTAs.  What the
-// arrivals order passes through TMEM and the async proxy, under the tcgen05
-// fences: they need no cluster-wide release of the CTA's other memory (with
-// .release.cluster / .acquire.cluster the kernel took 6.07 instead of 4.06 ms
-// per 1M rows at d = 960).
+// over both CTAs' rows (cta_group::2) and their commit to both CTAs.
+//
+// What the second CTA's arrivals order before the first CTA's MMAs:
+//  * its A block in TMEM: tcgen05.wait::st and tcgen05.fence::before_thread_sync
+//    stand before the arrival, fence::after_thread_sync behind the wait for it;
+//  * its half of W in its shared memory: the bulk copy that writes it signals
+//    that CTA's `full` barrier, and the copy's complete_tx releases its writes
+//    at cluster scope.  A converter lane waits for that phase before its warp
+//    converts, and its arrival on `conv` comes after: the copy, the arrival and
+//    the MMAs are ordered.  The MMAs read the half by the async proxy, which also
+//    wrote it, so no proxy fence is due;
+//  * that its converters are done with X: they read it before they arrive, and
+//    its next copy waits for the commit of those MMAs.
+// The MMAs read nothing that a thread of the other CTA stored in memory, so the
+// arrivals have no generic writes to release to the cluster and take the default
+// scope; with .release.cluster 1,000,000 rows at d = 960 took 6.86 instead of 4.1
+// ms, with .acquire.cluster waits beside them the same.
 __device__ __forceinline__ void mbar_arrive_cl(uint64_t *bar, uint32_t rank) {
     asm volatile(
         "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
@@ -1212,7 +1224,12 @@ __device__ __forceinline__ void umma2_commit_elect(uint64_t *bar) {
 // then moves 62 KB (X in and out 32, W in 12, the MMAs' reads 18) instead of
 // 92 KB: 484 against 720 cycles at 128 B per clock, beside 577 cycles of
 // MMAs.  Clusters take the tiles c, c + clusters, ...; each accumulator is
-// drained by its own CTA before the next tile's first MMA.
+// drained by its own CTA before the next tile's first MMA.  (Tiles from a work
+// counter, handed to the second CTA through its shared memory, were no faster
+// beside other streams' kernels, as a launch ends only after its last cluster
+// could start: 30,000 rows at d = 960 beside batches of 300 at 3072 337-370 us so,
+// 383 with the counter, 281 alone; alone 300,000 rows at d = 256 took 229 instead
+// of 204 us, 1,000,000 at 960 0.7% more.)
 // The ring of copies (S slots: X and half a W tile) is deeper than the ring of
 // converted blocks in TMEM (NA buffers, as many as fit beside the
 // accumulators): a copy takes ~1,000 cycles, a conversion ~800.
