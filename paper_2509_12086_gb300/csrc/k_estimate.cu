@@ -222,6 +222,16 @@ __device__ __forceinline__ int step_coord(int words, int step, int t, int i) {
     return at + ((words & 2) ? 128 : 0) + 16 * t + 4 * k + r + 8 * hi;
 }
 
+// A scaled coordinate's parts: the nearest integer (multiple of an FP16 unit in
+// the last place above 2048), and 4096 times what it leaves, in FP16.
+__device__ __forceinline__ float split_hi(float y) {
+    // 1.5 * 2^23 times that unit, whose sum with y rounds it off
+    const uint32_t e = max(__float_as_uint(fabsf(y)) >> 23, 137u);
+    const float m = __uint_as_float((e + 13u) << 23 | 0x400000u);
+    return (y + m) - m;
+}
+__device__ __forceinline__ float split_lo(float y, float hi) { return (y - hi) * 4096.f; }
+
 // B fragments of four queries (block x: column group pass * NT + nt) and one
 // segment (block y): entry ((pass * steps + step) * NT + nt) * 32 + lane holds
 // the four FP16 values of column lane / 4 (query 4 (pass * NT + nt) + column / 2,
@@ -230,56 +240,82 @@ __device__ __forceinline__ int step_coord(int words, int step, int t, int i) {
 // wstart[((pass * windows + window) * NT + nt) * 4 + query], and per segment
 // qseg[((pass * segments + segment) * NT + nt) * 4 + query]: the inverse scale and
 // what completes <u, q>, sum hi and -(2^b - 1) sum lo / 4096.
-constexpr int kSplitPieces = 1024;  // pieces whose sums are held at a time
-constexpr int kSplitWindows = 64;
-__global__ void __launch_bounds__(256)
+// The first block z of a segment forms the sums and the others share its K steps
+// (one block does both); each needs the scales, for which it reads the segment
+// once.  Bound by the
+// latency of those reads and sums: 5.8 us for a 960-long segment, 7.5 for 3,072
+// (17.7 with eight warps a block that read one piece at a time; under ncu).
+constexpr int kSplitPieces = 512;  // pieces whose sums are held at a time
+constexpr int kSplitWarps = 16;
+// Four sums over a warp's lanes; lane l gets sum l / 16 + 2 (l / 8 % 2).
+__device__ __forceinline__ float warp_sums(const float (&a)[4], int lane) {
+    const bool u = lane & 16, v = lane & 8;
+    const float b0 = (u ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, u ? a[0] : a[1], 16);
+    const float b1 = (u ? a[3] : a[2]) + __shfl_xor_sync(0xffffffffu, u ? a[2] : a[3], 16);
+    float c = (v ? b1 : b0) + __shfl_xor_sync(0xffffffffu, v ? b0 : b1, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+    return c;
+}
+__global__ void __launch_bounds__(32 * kSplitWarps)
 k_query_split(const float *__restrict__ qrot, int64_t nq, int dk,
               const __grid_constant__ SegTable t, int steps, int NT, int windows,
               uint2 *__restrict__ bfrag, float *__restrict__ wstart, float4 *__restrict__ qseg) {
-    __shared__ float piece[4][kSplitPieces];
-    __shared__ float part[kSplitWindows][8][8];
-    __shared__ float wmax[8], s_scale[4], s_inverse[4];
+    __shared__ float piece[2][4][kSplitPieces];
+    __shared__ float s_max[kSplitWarps], s_l1[4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t group = blockIdx.x, pass = group / NT, q0 = 4 * group;
-    const int nt = (int)(group % NT);
-    const int s = blockIdx.y;
+    const int nt = (int)(group % NT), s = blockIdx.y;
     const int len = t.s[s].len, words = t.s[s].words, bits = t.s[s].bits;
     const float *src = qrot + q0 * dk + t.s[s].off;
-    // ---- the scales: warp w takes the pieces of query w % 4 in turn
+    // warp w reads the pieces w / 4, w / 4 + 4, ... of query w % 4, four at a time
+    // (P to a window)
     const int pieces = (words + 1) / 2, full = words >> 2;
     const int P = bits <= kNarrow ? pieces : window_pieces(bits), nwin = (pieces + P - 1) / P;
+    const int wq = warp & 3;
+    const bool wlive = q0 + wq < nq;
+    const int which = (lane >> 4) | ((lane >> 3) & 1) << 1;  // warp_sums' of the lane
+    auto fetch = [&](int p0, float (&x)[4][4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int pi = p0 + 4 * k;
+                const int c = pi < 2 * full ? (4 * (pi >> 1) + j) * 64 + (pi & 1) * 32 + lane
+                                            : 256 * full + (pi - 2 * full) * 128 + 32 * j + lane;
+                x[k][j] = wlive && c < len ? __ldg(src + (int64_t)wq * dk + c) : 0.f;
+            }
+    };
+    auto warp_sum = [](float a) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        return a;
+    };
+    // ---- the scales
     {
-        const int b = warp & 3;
-        const float *p = src + (int64_t)b * dk;
-        const bool live = q0 + b < nq;
-        float mx = 0.f, l1 = 0.f;  // of lane 0 .. 31's windows
+        float mx = 0.f, l1 = 0.f;
         for (int p0 = 0; p0 < pieces; p0 += kSplitPieces) {
             const int pn = min(kSplitPieces, pieces - p0);
-#pragma unroll 4
-            for (int i = warp >> 2; i < pn; i += 2) {
-                const int pi = p0 + i;
-                float a = 0.f;
+            for (int i = warp >> 2; i < pn; i += 16) {
+                float x[4][4], a[4];
+                fetch(p0 + i, x);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int c = pi < 2 * full
-                                      ? (4 * (pi >> 1) + j) * 64 + (pi & 1) * 32 + lane
-                                      : 256 * full + (pi - 2 * full) * 128 + 32 * j + lane;
-                    const float v = live && c < len ? fabsf(__ldg(p + c)) : 0.f;
-                    a += v;
-                    mx = fmaxf(mx, v);
+                for (int k = 0; k < 4; ++k) {
+                    a[k] = (fabsf(x[k][0]) + fabsf(x[k][1])) + (fabsf(x[k][2]) + fabsf(x[k][3]));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) mx = fmaxf(mx, fabsf(x[k][j]));
                 }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                if (lane == 0) piece[b][i] = a;
+                const float c = warp_sums(a, lane);
+                if ((lane & 7) == 0 && i + 4 * which < pn) piece[0][wq][i + 4 * which] = c;
             }
             __syncthreads();
             if (warp < 4) {
                 if (nwin == 1) {
-                    for (int i = lane; i < pn; i += 32) l1 += piece[b][i];
+                    for (int i = lane; i < pn; i += 32) l1 += piece[0][wq][i];
                 } else {  // P divides kSplitPieces
                     for (int w = lane; w * P < pn; w += 32) {
                         float a = 0.f;
-                        for (int i = w * P; i < min(pn, w * P + P); ++i) a += piece[b][i];
+                        for (int i = w * P; i < min(pn, w * P + P); ++i) a += piece[0][wq][i];
                         l1 = a > l1 || a != a ? a : l1;  // a NaN stays
                     }
                 }
@@ -292,74 +328,88 @@ k_query_split(const float *__restrict__ qrot, int64_t nq, int dk,
             const float o = __shfl_xor_sync(0xffffffffu, l1, off);
             l1 = nwin == 1 ? l1 + o : o > l1 || o != o ? o : l1;
         }
-        if (lane == 0) wmax[warp] = mx;
-        __syncthreads();
-        if (warp < 4 && lane == 0) {
-            const int e = scale_exponent(l1, fmaxf(wmax[b], wmax[b + 4]), bits, min(len, 128 * P));
-            s_scale[b] = scalbnf(1.f, e);
-            s_inverse[b] = scalbnf(1.f, -e);
-        }
+        if (lane == 0) s_max[warp] = mx;
+        if (lane == 0 && warp < 4) s_l1[warp] = l1;
         __syncthreads();
     }
-    // ---- the columns, a K step per warp, and their sums by windows: G warps to
-    // a window
-    int G = 8;
-    while (G > 1 && nwin * G > 8) G >>= 1;
-    const int wg = warp / G, wi = warp % G;
+    auto exponent = [&](int b) {
+        const float mx = fmaxf(fmaxf(s_max[b], s_max[b + 4]), fmaxf(s_max[b + 8], s_max[b + 12]));
+        return scale_exponent(s_l1[b], mx, bits, min(len, 128 * P));
+    };
+    // ---- the sums
+    if (blockIdx.z == 0) {
+        const float scale = scalbnf(1.f, exponent(wq));
+        const float start = -(float)(1 << (bits - 1)) * 0x1p-24f;
+        float hi = 0.f, lo = 0.f;
+        float *ws = wstart + (pass * windows + t.s[s].window) * NT * 4 + nt * 4 + wq;
+        for (int p0 = 0; p0 < pieces; p0 += kSplitPieces) {
+            const int pn = min(kSplitPieces, pieces - p0);
+            for (int i = warp >> 2; i < pn; i += 16) {
+                float x[4][4], a[4], b[4];
+                fetch(p0 + i, x);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    a[k] = b[k] = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float y = x[k][j] * scale, r = split_hi(y);
+                        a[k] += r;
+                        b[k] += __half2float(__float2half_rn(split_lo(y, r)));
+                    }
+                }
+                const float ca = warp_sums(a, lane), cb = warp_sums(b, lane);
+                if ((lane & 7) == 0 && i + 4 * which < pn) {
+                    piece[0][wq][i + 4 * which] = ca;
+                    piece[1][wq][i + 4 * which] = cb;
+                }
+            }
+            __syncthreads();
+            if (warp < 4)
+                for (int w = lane; w * P < pn || (nwin == 1 && w < pn); w += 32) {
+                    // (one window: a piece each)
+                    const int i0 = nwin == 1 ? w : w * P, i1 = nwin == 1 ? w + 1 : min(pn, w * P + P);
+                    float a = 0.f;  // integers below 2^24, exact in any order
+                    for (int i = i0; i < i1; ++i) {
+                        a += piece[0][wq][i];
+                        lo += piece[1][wq][i];
+                    }
+                    hi += a;
+                    if (nwin > 1) ws[(int64_t)(p0 / P + w) * NT * 4] = start * a;
+                }
+            __syncthreads();
+        }
+        if (warp < 4) {
+            hi = warp_sum(hi);
+            lo = warp_sum(lo);
+            if (lane == 0) {
+                if (nwin == 1) ws[0] = start * hi;
+                qseg[((pass * gridDim.y + s) * NT + nt) * 4 + wq] =
+                    make_float4(scalbnf(1.f, -exponent(wq)), hi,
+                                -(float)((1 << bits) - 1) * 0x1p-12f * lo, 0.f);
+            }
+        }
+    }
+    // ---- the columns, a K step to a warp
+    const int sharing = max(1, (int)gridDim.z - 1), slice = gridDim.z > 1 ? (int)blockIdx.z - 1 : 0;
+    if (slice < 0) return;
     const int b = lane >> 3;
     const bool lo = (lane >> 2) & 1, live = q0 + b < nq;
-    const float scale = s_scale[b];
+    const float scale = scalbnf(1.f, exponent(b));
     const float *p = src + (int64_t)b * dk;
     uint2 *out = bfrag + ((pass * steps + t.s[s].step) * NT + nt) * 32 + lane;
-    float total = 0.f;  // of column threadIdx.x < 8 over the segment
-    for (int v0 = 0; v0 < nwin; v0 += kSplitWindows) {
-        const int vn = min(kSplitWindows, nwin - v0);
-        for (int v = wg; v < vn; v += 8 / G) {
-            const int first = 8 * P * (v0 + v), last = min(4 * words, first + 8 * P);
-            float sum = 0.f;
-#pragma unroll 4
-            for (int step = first + wi; step < last; step += G) {
-                __half h[4];
+#pragma unroll 2
+    for (int step = slice * kSplitWarps + warp; step < 4 * words; step += kSplitWarps * sharing) {
+        float x[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int c = step_coord(words, step, lane & 3, i);
-                    float x = 0.f;
-                    if (live && c < len) {
-                        const float y = __ldg(p + c) * scale;
-                        const float r = fabsf(y) < 2048.f ? rintf(y) : __half2float(__float2half_rn(y));
-                        x = lo ? (y - r) * 4096.f : r;
-                    }
-                    h[i] = __float2half_rn(x);
-                    sum += __half2float(h[i]);
-                }
-                uint2 o;
-                o.x = (uint32_t)__half_as_ushort(h[0]) | (uint32_t)__half_as_ushort(h[1]) << 16;
-                o.y = (uint32_t)__half_as_ushort(h[2]) | (uint32_t)__half_as_ushort(h[3]) << 16;
-                out[(int64_t)step * NT * 32] = o;
-            }
-            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-            if ((lane & 3) == 0) part[v][wi][lane >> 2] = sum;
+        for (int i = 0; i < 4; ++i) {
+            const int c = step_coord(words, step, lane & 3, i);
+            const float y = live && c < len ? __ldg(p + c) * scale : 0.f;
+            const float r = split_hi(y);
+            x[i] = lo ? split_lo(y, r) : r;
         }
-        __syncthreads();
-        const float start = -(float)(1 << (bits - 1)) * 0x1p-24f;
-        for (int e = threadIdx.x; e < 8 * vn; e += 256) {
-            const int v = e >> 3, c = e & 7;
-            float sum = 0.f;  // hi: integers below 2^24, in any order exact
-            for (int w = 0; w < G; ++w) sum += part[v][w][c];
-            part[v][0][c] = sum;
-            if (!(c & 1)) wstart[((pass * windows + t.s[s].window + v0 + v) * NT + nt) * 4 + (c >> 1)] = start * sum;
-        }
-        __syncthreads();
-        if (threadIdx.x < 8)
-            for (int v = 0; v < vn; ++v) total += part[v][0][threadIdx.x];
-        __syncthreads();
-    }
-    if (warp == 0) {
-        const float lo_sum = __shfl_down_sync(0xffffffffu, total, 1);
-        if (lane < 8 && !(lane & 1))
-            qseg[((pass * gridDim.y + s) * NT + nt) * 4 + (lane >> 1)] = make_float4(
-                s_inverse[lane >> 1], total, -(float)((1 << bits) - 1) * 0x1p-12f * lo_sum, 0.f);
+        const __half2 h0 = __floats2half2_rn(x[0], x[1]), h1 = __floats2half2_rn(x[2], x[3]);
+        out[(int64_t)step * NT * 32] =
+            make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
     }
 }
 
@@ -573,9 +623,14 @@ __device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], i
             at -= stride;
         }
     };
-    if (pieces > 0) fetch(0);
+    // a staged record is read when it is needed, as the registers that hold the
+    // next piece cost warps or spills (100 queries x 100K at 8 b/dim read ahead
+    // 717 us, so 675; 1 x 1M at 4 b/dim 278 and 271)
+    constexpr bool kAhead = !SM;
+    if (kAhead && pieces > 0) fetch(0);
 #pragma unroll 1
     for (int i = 0; i < pieces; ++i) {
+        if constexpr (!kAhead) fetch(i);
         if (partial) {
             const int left = len - (int)piece_at(i) * 8;
             const uint32_t keep = left >= 32 ? ~0u : left <= 0 ? 0u : (1u << left) - 1u;
@@ -595,7 +650,7 @@ __device__ __forceinline__ void run_segment(const uint8_t *const (&rp)[MT][2], i
                 cd[mt][h].split(nx[mt][h]);
                 S2[mt][h] = cd[mt][h].sum2(S2[mt][h]);
             }
-        if (i + 1 < pieces) fetch(i + 1);
+        if (kAhead && i + 1 < pieces) fetch(i + 1);
         window_ends(i);
         run_steps<NP, NT, MT, 8>(cd, b, acc);
         b += 8 * NT * 32;
@@ -678,10 +733,8 @@ __host__ __device__ constexpr size_t table_bytes(int windows, int segments, int 
     return (size_t)(windows + 4 * segments) * 4 * NT * sizeof(float);
 }
 
-// Warps of a block of the staged form: with 24 (80 registers a thread) up to
-// four B tiles spill, 10 queries x 100K staged bounds at 8 b/dim 140 us, with 20
-// (96) 131.
-__host__ __device__ constexpr int staged_warps(int NT) { return NT <= 4 ? 20 : 12; }
+// Warps of a block of the staged form: as many as their registers allow.
+__host__ __device__ constexpr int staged_warps(int NT) { return NT <= 4 ? 24 : 12; }
 
 // A warp takes tiles of 16 MT vectors; the block's NT B columns (4 NT queries
 // of pass blockIdx.y) stay in shared memory (BS) for all of its tiles.
@@ -691,7 +744,7 @@ __host__ __device__ constexpr int staged_warps(int NT) { return NT <= 4 ? 20 : 1
 // HBM round trip at the start of every segment; the other warps of the SM
 // cover the copy.
 // Bound by the instructions of the decode: 1 query x 1M records of 480 B 4,350 ->
-// 279 us, 100 x 100K 22,600 -> 231 us, against a warp per (query, vector) that
+// 271 us, 100 x 100K 22,600 -> 227 us, against a warp per (query, vector) that
 // decoded a bit per plane and lane.
 // Measured on the way: decode to FP16 integers by two more FP16 operations
 // per pair 405 us, |u|^2 from two more products per step (their diagonals)
@@ -1097,9 +1150,19 @@ saq_status launch_estimate(const saq_model *m, const uint8_t *codes, const float
     } else {
         saq_status st = launch_query_rot(m, Q, nq, m->d_W, w.qrot, w.qn2, s);
         if (st != SAQ_OK) return st;
+        // a few queries: blocks that share a segment's steps, a step per warp at
+        // most, up to two blocks to an SM
+        int dev = 0, sms = 0, steps = 0;
+        SAQ_CUDA_CHECK(cudaGetDevice(&dev));
+        SAQ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        for (const KeptSeg &k : m->kept) steps = std::max(steps, 4 * k.words);
+        const int64_t blocks = p.passes * p.NT * nk;
+        const int64_t share = std::max<int64_t>(
+            1, std::min<int64_t>(1 + (steps + kSplitWarps - 1) / kSplitWarps, 2 * sms / blocks));
         {
             LaunchTimer lt_(kKindOther, s);
-            k_query_split<<<dim3((unsigned)(p.passes * p.NT), (unsigned)nk), 256, 0, s>>>(
+            k_query_split<<<dim3((unsigned)(p.passes * p.NT), (unsigned)nk, (unsigned)share),
+                            32 * kSplitWarps, 0, s>>>(
                 w.qrot, nq, m->dk, t, p.steps, p.NT, windows, w.bfrag, w.wstart, w.qseg);
         }
         note_launches();
