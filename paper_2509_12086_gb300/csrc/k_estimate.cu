@@ -1024,8 +1024,11 @@ saq_status launch_form(const EstArgs &a, const SegTable &t, const EstPlan &p, in
     const int64_t tiles = (a.n + 16 * MT - 1) / (16 * MT);
     for (int64_t p0 = 0; p0 < p.passes; p0 += 65535) {
         const int64_t np = std::min<int64_t>(65535, p.passes - p0);
-        // the passes share the SMs; a block keeps its B columns over its tiles
-        const int64_t each = std::max<int64_t>(1, ((int64_t)sms * std::max(1, per_sm) + np - 1) / np);
+        // the passes share the SMs; a block keeps its B columns over its tiles.
+        // No more blocks than are resident at once: seven passes of 22 on 152
+        // SMs left two for a wave of their own (100 queries x 100K at 8 b/dim
+        // 675 -> 375 us)
+        const int64_t each = std::max<int64_t>(1, (int64_t)sms * std::max(1, per_sm) / np);
         // few tiles: as many blocks as there are SMs to take them
         int w = warps;
         if (SM) w = (int)std::max<int64_t>(4, std::min<int64_t>(w, (tiles + each - 1) / each));
