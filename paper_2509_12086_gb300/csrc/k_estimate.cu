@@ -61,13 +61,13 @@ struct SegTable {
 
 // ------------------------------------------------------------ the queries
 // out[q * dk + j] = <M_j, q_r - c> for the rows M_j of a dk x d matrix, and with
-// qn2 also |q_r - c|^2.  A warp computes
-// CPW columns for QB queries: its lanes split the d coordinates (the rows of
-// M are read once, coalesced, and each value meets QB centred queries in
-// shared memory), so that a single query spreads over dk warps (d = 960: 8.5
-// us; on the 128 x 128 tiles of the row projection, eight blocks, 207 us).  Only
-// the coordinates there are get staged (with 1,024 whatever d is: 16,000 queries
-// at d = 128 79 -> 47 us, 8,000 at 1536 1,609 -> 1,264, 8,000 at 960 622 -> 611).
+// qn2 also |q_r - c|^2.  A warp computes CPW columns for QB queries: its lanes
+// split the d coordinates (the rows of M are read once, coalesced, and each
+// value meets QB centred queries in shared memory), so that a single query
+// spreads over dk warps (d = 960: 8.5 us; on the 128 x 128 tiles of the row
+// projection, eight blocks, 207 us).  Only the coordinates there are get staged
+// (with 1,024 whatever d is: 16,000 queries at d = 128 79 -> 47 us, 8,000 at 1536
+// 1,609 -> 1,264, 8,000 at 960 622 -> 611).
 // The row projection's tiles, whose sums run over all coordinates in one lane,
 // are as fast at 16,000 queries of 128 coordinates (44 us) and faster beyond
 // (64,000: 111 against 214).
@@ -241,10 +241,10 @@ __device__ __forceinline__ float split_lo(float y, float hi) { return (y - hi) *
 // qseg[((pass * segments + segment) * NT + nt) * 4 + query]: the inverse scale and
 // what completes <u, q>, sum hi and -(2^b - 1) sum lo / 4096.
 // The first block z of a segment forms the sums and the others share its K steps
-// (one block does both); each needs the scales, for which it reads the segment
-// once.  Bound by the
-// latency of those reads and sums: 5.8 us for a 960-long segment, 7.5 for 3,072
-// (17.7 with eight warps a block that read one piece at a time; under ncu).
+// (a block that is alone does both); each needs the scales, for which it reads the
+// segment once.  Bound by the latency of those reads and sums: 5.8 us for a
+// 960-long segment, 7.5 for 3,072 (17.7 with eight warps a block that read one
+// piece at a time; under ncu).
 constexpr int kSplitPieces = 512;  // pieces whose sums are held at a time
 constexpr int kSplitWarps = 16;
 // Four sums over a warp's lanes; lane l gets sum l / 16 + 2 (l / 8 % 2).
